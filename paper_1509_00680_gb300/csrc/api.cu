@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "device_util.cuh"
+#include "fix64.cuh"
 #include "gps_internal.h"
 #include "kernels.h"
 
@@ -378,7 +379,7 @@ struct Shape {
     PassGeom g;
     FftSched fx, fy, fz;
   } sp[3];                    // per spectrum precision (Spec), set by the autotuner
-  double2 *twx64 = nullptr, *twy64 = nullptr, *twz64 = nullptr;
+  i64c *twx64 = nullptr, *twy64 = nullptr, *twz64 = nullptr;   // Q62 digits
   float2 *twx32 = nullptr, *twy32 = nullptr, *twz32 = nullptr;
   dfc *twxdf = nullptr, *twydf = nullptr, *twzdf = nullptr;
   double* table = nullptr;
@@ -388,38 +389,40 @@ struct Shape {
   DevMem mem;
 };
 
-int batch_lines(int L, int units) { return default_lines(L, units, sizeof(double2)); }
+int batch_lines(int L, int units) { return default_lines(L, units, sizeof(i64c)); }
 
-void upload_twiddles(Shape* S, int L, double2** t64, float2** t32, dfc** tdf) {
-  std::vector<double2> h64(L);
+void upload_twiddles(Shape* S, int L, i64c** t64, float2** t32, dfc** tdf) {
+  std::vector<i64c> h64(L);
   std::vector<float2> h32(L);
   std::vector<dfc> hdf(L);
   for (int m = 0; m < L; ++m) {
     const long double ang = 2.0L * 3.141592653589793238462643383279502884L * m / L;
     const long double c = cosl(ang), s = -sinl(ang);
-    h64[m].x = (double)c;
-    h64[m].y = (double)s;
-    h32[m].x = (float)h64[m].x;
-    h32[m].y = (float)h64[m].y;
+    h64[m].x = fx(q62_digits(llrintl(c * 4611686018427387904.0L)));
+    h64[m].y = fx(q62_digits(llrintl(s * 4611686018427387904.0L)));
+    h32[m].x = (float)(double)c;
+    h32[m].y = (float)(double)s;
     // double-float split taken from the long double value
     const float cx = (float)c, sy = (float)s;
     hdf[m].x = df(cx, (float)(c - (long double)cx));
     hdf[m].y = df(sy, (float)(s - (long double)sy));
   }
-  // FP32 and df64 tables carry, after the plain table, the per-stage layouts
-  // of the register-resident column passes (zeros where L is not served).
+  // After the plain table come the per-stage layouts of the register-resident
+  // passes (zeros where L is not served).
   std::vector<int> idx(2 * (size_t)L, 0);
   const bool col = col_stage_twiddle_index(L, idx.data());
+  h64.resize(3 * (size_t)L);
   h32.resize(3 * (size_t)L);
   hdf.resize(3 * (size_t)L);
   for (size_t i = 0; i < 2 * (size_t)L; ++i) {
+    h64[L + i] = col ? h64[idx[i]] : i64c{fx(0), fx(0)};
     h32[L + i] = col ? h32[idx[i]] : float2{0.f, 0.f};
     hdf[L + i] = col ? hdf[idx[i]] : dfc{df(0.f, 0.f), df(0.f, 0.f)};
   }
-  *t64 = S->mem.alloc<double2>(L);
+  *t64 = S->mem.alloc<i64c>(3 * (size_t)L);
   *t32 = S->mem.alloc<float2>(3 * (size_t)L);
   *tdf = S->mem.alloc<dfc>(3 * (size_t)L);
-  ck(cudaMemcpy(*t64, h64.data(), L * sizeof(double2), cudaMemcpyHostToDevice));
+  ck(cudaMemcpy(*t64, h64.data(), 3 * (size_t)L * sizeof(i64c), cudaMemcpyHostToDevice));
   ck(cudaMemcpy(*t32, h32.data(), 3 * (size_t)L * sizeof(float2), cudaMemcpyHostToDevice));
   ck(cudaMemcpy(*tdf, hdf.data(), 3 * (size_t)L * sizeof(dfc), cudaMemcpyHostToDevice));
 }
@@ -526,6 +529,7 @@ std::shared_ptr<Shape> build_shape(const gps_grid* gr, cudaStream_t st) {
   S->periodic = gr->bc == GPS_BC_PERIODIC;
   S->inv_p = 1.0 / ((double)S->Px * S->Py * S->Pz);
   PassGeom& g = S->g;
+  g = PassGeom{};
   g.nx = gr->nx; g.ny = gr->ny; g.nz = gr->nz;
   g.Px = S->Px; g.Py = S->Py; g.Pz = S->Pz; g.Hx = S->Hx; g.Hp = S->Hp;
   g.nrows = gr->ny * gr->nz;
@@ -602,7 +606,7 @@ struct Pool {
   int pstride = 0;
   Fields f{};
   double *own_rho = nullptr, *own_eps = nullptr, *own_phi = nullptr, *own_gam = nullptr;
-  double2* W64 = nullptr;
+  i64c* W64 = nullptr;        // FP64 or df64 spectrum
   float2* W32 = nullptr;
   double *partials = nullptr, *partials2 = nullptr, *partials3 = nullptr;
   SlotState* st = nullptr;
@@ -648,7 +652,7 @@ struct Pool {
 
 size_t slot_bytes(const Shape& S) {
   const size_t wn = (size_t)S.Hp * S.Py * S.grid.nz;
-  return 18 * S.n * sizeof(double) + S.n * sizeof(float) + wn * (sizeof(double2) + sizeof(float2)) +
+  return 18 * S.n * sizeof(double) + S.n * sizeof(float) + wn * (sizeof(i64c) + sizeof(float2)) +
          3 * 4096 * sizeof(double);
 }
 
@@ -692,7 +696,7 @@ std::unique_ptr<Pool> make_pool(std::shared_ptr<Shape> shape, int cap, bool own_
   f.dphi = P->mem.alloc<double>(N);
   f.src = P->mem.alloc<double>(N);
   f.tmp = P->mem.alloc<double>(N);
-  P->W64 = P->mem.alloc<double2>(P->wn * cap);
+  P->W64 = P->mem.alloc<i64c>(P->wn * cap);
   P->W32 = P->mem.alloc<float2>(P->wn * cap);
   P->partials = P->mem.alloc<double>((size_t)P->pstride * cap);
   P->partials2 = P->mem.alloc<double>((size_t)P->pstride * cap);
@@ -729,7 +733,7 @@ Batch batch_of(Pool& P, int phase, int prec) {
 }
 
 template <typename V> constexpr int spec_of() {
-  return std::is_same<V, double2>::value ? SPEC_FP64 : std::is_same<V, float2>::value ? SPEC_FP32 : SPEC_DF64;
+  return std::is_same<V, i64c>::value ? SPEC_FP64 : std::is_same<V, float2>::value ? SPEC_FP32 : SPEC_DF64;
 }
 
 // One spectrum pipeline (five passes) for the slots of `b`.
@@ -737,10 +741,10 @@ template <typename V>
 void pipeline(Pool& P, const Batch& b, PipeArgs a, cudaStream_t st) {
   const Shape& S = *P.shape;
   const V *twx, *twy, *twz;
-  if constexpr (std::is_same<V, double2>::value) {
-    twx = reinterpret_cast<const V*>(S.twx64);
-    twy = reinterpret_cast<const V*>(S.twy64);
-    twz = reinterpret_cast<const V*>(S.twz64);
+  if constexpr (std::is_same<V, i64c>::value) {
+    twx = S.twx64;
+    twy = S.twy64;
+    twz = S.twz64;
     a.W = P.W64;
   } else if constexpr (std::is_same<V, dfc>::value) {
     twx = S.twxdf;
@@ -858,10 +862,10 @@ void tune_spec(Shape& S, cudaStream_t st) {
   auto hit = g_tune.find(key);
   if (hit == g_tune.end()) {
     const V *twx, *twy, *twz;
-    if constexpr (std::is_same<V, double2>::value) {
-      twx = reinterpret_cast<const V*>(S.twx64);
-      twy = reinterpret_cast<const V*>(S.twy64);
-      twz = reinterpret_cast<const V*>(S.twz64);
+    if constexpr (std::is_same<V, i64c>::value) {
+      twx = S.twx64;
+      twy = S.twy64;
+      twz = S.twz64;
     } else if constexpr (std::is_same<V, dfc>::value) {
       twx = S.twxdf;
       twy = S.twydf;
@@ -904,10 +908,10 @@ void tune_spec(Shape& S, cudaStream_t st) {
     best.fy = S.fy;
     best.fz = S.fz;
     // passes served by the register-resident kernels (fixed tiling, compile-time radix plan)
-    const bool f64 = std::is_same<V, double2>::value;
-    const bool fixx = std::is_same<V, dfc>::value && col_pass_supported(S.Px);
-    const bool fixy = !f64 && col_pass_supported(S.Py);
-    const bool fixz = !f64 && col_pass_supported(S.Pz);
+    const bool f64 = std::is_same<V, i64c>::value;
+    const bool fixx = !std::is_same<V, float2>::value && col_pass_supported(S.Px);
+    const bool fixy = col_pass_supported(S.Py);
+    const bool fixz = col_pass_supported(S.Pz);
     // radix orders: 8s first, 8s last, 4s, and for FP64 16s first
     const int norders = f64 ? 4 : 3;
     // x passes: lines per CTA and radix order of Px
@@ -958,7 +962,7 @@ void tune_spec(Shape& S, cudaStream_t st) {
         if (t < tbest) { tbest = t; best.g.tile_z = tile; best.fz = fz; }
       }
     // column kernels: the TMA-staged z pass as one more candidate
-    if (fixz && g_z_kernel != 0) {
+    if (fixz && !f64 && g_z_kernel != 0) {
       PassGeom g = best.g;
       g.z_tma = 1;
       const float t = time_launch([&] { launch_z<V>(g, best.fz, twz, b, a, 1, st); }, st);
@@ -978,7 +982,7 @@ void tune_spec(Shape& S, cudaStream_t st) {
 // needed: setup of periodic q and the certificate run in FP64).  Must run
 // outside stream capture.
 void ensure_tuned(Shape& S, bool fp32, bool df64, cudaStream_t st) {
-  tune_spec<double2>(S, st);
+  tune_spec<i64c>(S, st);
   if (fp32) tune_spec<float2>(S, st);
   if (df64) tune_spec<dfc>(S, st);
 }
@@ -993,7 +997,7 @@ void launch_setup_group(Pool& P, cudaStream_t st) {
     a.out = P.f.q;
     a.out_scale = P.f.sq;
     a.table = S.lap;
-    pipeline<double2>(P, b, a, st);
+    pipeline<i64c>(P, b, a, st);
   } else {
     const int per_xy = S.grid.bc == GPS_BC_SURFACE ? 1 : 0;   // surface: x, y wrap; z free
     const int per_z = S.grid.bc == GPS_BC_WIRE ? 1 : 0;       // wire: z wraps; x, y free
@@ -1033,7 +1037,7 @@ void launch_round(Pool& P, int m, bool setup, bool init, cudaStream_t st) {
   const Batch bidf = batch_of(P, PH_ITER, SPEC_DF64);
   const Batch bi = batch_of(P, PH_ITER, -1);
   for (int i = 0; i < m; ++i) {
-    if (P.has_fp64) pipeline<double2>(P, bi64, it, st);
+    if (P.has_fp64) pipeline<i64c>(P, bi64, it, st);
     if (P.has_df64) pipeline<dfc>(P, bidf, it, st);
     if (P.has_mixed) pipeline<float2>(P, bi32, it, st);
     timed(5, bi, st, [&](const Batch& bb) { launch_update_p(bb, f, n, periodic, ns, st); });
@@ -1055,7 +1059,7 @@ void launch_round(Pool& P, int m, bool setup, bool init, cudaStream_t st) {
     c.table32 = S.table32;
     c.tabledf = S.tabledf;
     c.slot_k0 = 1;
-    pipeline<double2>(P, bc, c, st);
+    pipeline<i64c>(P, bc, c, st);
     launch_fp_residual(bc, f, n, periodic, ns, st);
   }
 }
@@ -1672,13 +1676,13 @@ int solve_comparison(Pool& P, const double* rho, const double* eps, double* phi,
       pa.in = w.c;
       pa.in_scale = nullptr;
       pa.out = phi;
-      pipeline<double2>(P, b, pa, st);
+      pipeline<i64c>(P, b, pa, st);
       prof(8, [&](const ScArgs& aa) { launch_sc_step(aa, st); });
     } else if (!m) {
       pa.in = r;
       pa.in_scale = w.isc;
       pa.out = v;
-      pipeline<double2>(P, b, pa, st);
+      pipeline<i64c>(P, b, pa, st);
       prof(8, [&](const ScArgs& aa) { launch_psd_av(aa, v, r, Av, 0, st); });
       prof(9, [&](const ScArgs& aa) { launch_psd_update(aa, phi, r, v, Av, phi, r, -1, st); });
     } else {
@@ -1686,7 +1690,7 @@ int solve_comparison(Pool& P, const double* rho, const double* eps, double* phi,
       pa.in = a.hist_r + (size_t)j * n;
       pa.in_scale = w.isc;
       pa.out = a.hist_v + (size_t)j * n;
-      pipeline<double2>(P, b, pa, st);
+      pipeline<i64c>(P, b, pa, st);
       DiisSlots sl{};
       sl.cnt = cnt;
       for (int q = 0; q < cnt; ++q) sl.slot[q] = (k - cnt + 1 + q) % m;
@@ -2047,7 +2051,7 @@ int gps_vacuum_solve(gps_ctx* ctx, const gps_grid* grid, const double* sigma, do
   a.table = P->shape->table;
   a.table32 = P->shape->table32;
   a.tabledf = P->shape->tabledf;
-  pipeline<double2>(*P, b, a, st);
+  pipeline<i64c>(*P, b, a, st);
   return finish(GPS_OK, st);
   GPS_GUARD_END
 }
@@ -2081,7 +2085,7 @@ int gps_precondition(gps_ctx* ctx, const gps_grid* grid, const double* s, const 
   }
   if (precision == GPS_MIXED) pipeline<float2>(*P, b, a, st);
   else if (precision == GPS_DF64) pipeline<dfc>(*P, b, a, st);
-  else pipeline<double2>(*P, b, a, st);
+  else pipeline<i64c>(*P, b, a, st);
   return finish(GPS_OK, st);
   GPS_GUARD_END
 }

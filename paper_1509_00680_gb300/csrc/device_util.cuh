@@ -135,7 +135,6 @@ struct __align__(16) dfc {
 };
 
 template <typename V> struct Real;
-template <> struct Real<double2> { using T = double; };
 template <> struct Real<float2> { using T = float; };
 template <> struct Real<dfc> { using T = df; };
 

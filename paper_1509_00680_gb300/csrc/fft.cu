@@ -20,6 +20,55 @@
 
 namespace gps {
 
+// Scales of the lines of a CTA (FP64 spectrum, see fix64.cuh), in shared
+// memory: an element of exponent e is shifted by base - e before the first
+// stage and by rem before the first stage whose product of radices passes
+// short_product(L); exp is the exponent of the transformed line.
+struct LineScales {
+  int *base, *rem, *exp;
+};
+// Up to 1024 points one shift before the first stage leaves the elements 50
+// bits and more; longer lines would lose more to it than FP64 rounding
+// (measured on white noise at 4096 points: 1.1e-15 against 3.3e-16), so they
+// are shifted for 64-point products first.
+__device__ __forceinline__ int short_product(int L) { return L > 1024 ? 64 : 512; }
+__device__ __forceinline__ int headroom(int L) { return L > 1024 ? kHeadroom - 3 : kHeadroom; }
+
+__device__ __forceinline__ i64c fx_scaled(i64c w, int base, int parity) {
+  const int sh = base - packed_exp(w);
+  return i64c{fx(shift_round(packed_man(w.x.v) - parity, sh)), fx(shift_round(packed_man(w.y.v) - parity, sh))};
+}
+
+// Scales of `nlines` lines of L packed values of which the first nin may be
+// nonzero: a warp per line; extra: bits kept free below 2^62.
+__device__ __forceinline__ void line_scales(const i64c* buf, int L, int ls, int nlines, int nin, int extra,
+                                            const LineScales& sc) {
+  const int lane = threadIdx.x & 31;
+  for (int line = threadIdx.x >> 5; line < nlines; line += blockDim.x >> 5) {
+    const i64c* src = buf + line * ls;
+    int em = -(1 << 28);
+    unsigned int sum = 0;
+    for (int j = lane; j < nin; j += 32) {
+      const i64c w = src[pidx<i64c>(j)];
+      const int e = packed_exp(w);
+      if (e > em) {
+        sum = (sum >> min(e - em, 31)) + 1u;
+        em = e;
+      }
+      sum += mag_part(w.x.v, w.y.v, em - e);
+    }
+    const int top = __reduce_max_sync(0xffffffffu, em);
+    sum = __reduce_add_sync(0xffffffffu, (sum >> min(top - em, 31)) + 1u);
+    if (lane == 0) {
+      const int shift = max(sum_shift(sum) + extra, 1), first = min(shift, headroom(L) + extra);
+      sc.base[line] = top + first;
+      sc.rem[line] = shift - first;
+      sc.exp[line] = top + shift;
+    }
+  }
+  __syncthreads();
+}
+
 // One Stockham stage over `nlines` lines of length L (line stride ls):
 // butterfly j gathers in[j + r L/R], twiddles by W_(Ns R)^(r k), k = j mod Ns,
 // and scatters to out[(j - k) R + k + r Ns].  Butterflies are dealt to the
@@ -31,9 +80,12 @@ namespace gps {
 // HALF (first stage only, Ns = 1): elements L/2.. of every line are the zero
 // padding, i.e. x[R/2..R-1] of every butterfly; they are neither read nor
 // used (Dft::run_half).
+// i64c: in the first stage the lines hold packed values, which it shifts to
+// the line's scale (sc.base); the stage that passes 512-point products takes
+// the rest of a long line's shift (sc.rem).
 template <typename V, int DIR, int R, bool FL, bool FS, bool HALF = false>
 __device__ __forceinline__ void stage(const V* __restrict__ in, V* __restrict__ out, int L, int Ns,
-                                      int ls, int nlines, const V* __restrict__ tw) {
+                                      int ls, int nlines, const V* __restrict__ tw, const LineScales& sc) {
   constexpr int P = 1 << PadShift<V>::v;
   const int nb = L / R;
   const int tstep = L / (Ns * R);
@@ -50,6 +102,22 @@ __device__ __forceinline__ void stage(const V* __restrict__ in, V* __restrict__ 
     const int s0 = pidx<V>(j);
 #pragma unroll
     for (int r = 0; r < (HALF ? R / 2 : R); ++r) x[r] = src[FL ? s0 + r * snb : pidx<V>(j + r * nb)];
+    if constexpr (std::is_same<V, i64c>::value) {
+      if (Ns == 1) {
+        const int base = sc.base[line];
+#pragma unroll
+        for (int r = 0; r < (HALF ? R / 2 : R); ++r) x[r] = fx_scaled(x[r], base, (j + r) & 1);
+      } else if (Ns <= short_product(L) && Ns * R > short_product(L)) {
+        const int rem = sc.rem[line];
+        if (rem > 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            x[r].x.v = shift_round(x[r].x.v - (r & 1), rem);
+            x[r].y.v = shift_round(x[r].y.v - (r & 1), rem);
+          }
+        }
+      }
+    }
     if (!HALF && k != 0) {
       const int step = tstep * k;
 #pragma unroll
@@ -77,21 +145,22 @@ __device__ __forceinline__ void stage(const V* __restrict__ in, V* __restrict__ 
 
 template <typename V, int DIR, int R>
 __device__ __forceinline__ void stage_any(const V* in, V* out, int L, int Ns, int ls, int nlines,
-                                          const V* tw) {
+                                          const V* tw, const LineScales& sc) {
   constexpr int P = 1 << PadShift<V>::v;
   const bool fl = (L / R) % P == 0, fs = Ns % P == 0;
-  if (fl && fs) stage<V, DIR, R, true, true>(in, out, L, Ns, ls, nlines, tw);
-  else if (fl) stage<V, DIR, R, true, false>(in, out, L, Ns, ls, nlines, tw);
-  else if (fs) stage<V, DIR, R, false, true>(in, out, L, Ns, ls, nlines, tw);
-  else stage<V, DIR, R, false, false>(in, out, L, Ns, ls, nlines, tw);
+  if (fl && fs) stage<V, DIR, R, true, true>(in, out, L, Ns, ls, nlines, tw, sc);
+  else if (fl) stage<V, DIR, R, true, false>(in, out, L, Ns, ls, nlines, tw, sc);
+  else if (fs) stage<V, DIR, R, false, true>(in, out, L, Ns, ls, nlines, tw, sc);
+  else stage<V, DIR, R, false, false>(in, out, L, Ns, ls, nlines, tw, sc);
 }
 
 // First stage (Ns = 1, so FS holds) of a line whose upper half is zero.
 template <typename V, int DIR, int R>
-__device__ __forceinline__ void stage_half(const V* in, V* out, int L, int ls, int nlines, const V* tw) {
+__device__ __forceinline__ void stage_half(const V* in, V* out, int L, int ls, int nlines, const V* tw,
+                                           const LineScales& sc) {
   constexpr int P = 1 << PadShift<V>::v;
-  if ((L / R) % P == 0) stage<V, DIR, R, true, false, true>(in, out, L, 1, ls, nlines, tw);
-  else stage<V, DIR, R, false, false, true>(in, out, L, 1, ls, nlines, tw);
+  if ((L / R) % P == 0) stage<V, DIR, R, true, false, true>(in, out, L, 1, ls, nlines, tw, sc);
+  else stage<V, DIR, R, false, false, true>(in, out, L, 1, ls, nlines, tw, sc);
 }
 
 // Full 1D transform of a batch of lines held in a; b is the ping-pong partner.
@@ -104,19 +173,19 @@ __device__ __forceinline__ void stage_half(const V* in, V* out, int L, int ls, i
 // axis pads n to 2n, and the first radix of every schedule is even).
 template <typename V, int DIR, int MR = 8, bool PRUNE = true>
 __device__ __forceinline__ V* fft_lines(V* a, V* b, const FftSched& s, int ls, int nlines, const V* tw,
-                                        int nin) {
+                                        int nin, const LineScales& sc) {
   V* in = a;
   V* out = b;
   for (int st = 0; st < s.nst; ++st) {
     const int R = s.radix[st], Ns = s.ns[st];
     if (PRUNE && st == 0 && 2 * nin == s.L && R % 2 == 0) {
       switch (R) {
-        case 2: stage_half<V, DIR, 2>(in, out, s.L, ls, nlines, tw); break;
-        case 4: stage_half<V, DIR, 4>(in, out, s.L, ls, nlines, tw); break;
+        case 2: stage_half<V, DIR, 2>(in, out, s.L, ls, nlines, tw, sc); break;
+        case 4: stage_half<V, DIR, 4>(in, out, s.L, ls, nlines, tw, sc); break;
         case 16:
-          if constexpr (MR == 16) stage_half<V, DIR, 16>(in, out, s.L, ls, nlines, tw);
+          if constexpr (MR == 16) stage_half<V, DIR, 16>(in, out, s.L, ls, nlines, tw, sc);
           break;
-        default: stage_half<V, DIR, 8>(in, out, s.L, ls, nlines, tw); break;
+        default: stage_half<V, DIR, 8>(in, out, s.L, ls, nlines, tw, sc); break;
       }
       __syncthreads();
       V* t = in;
@@ -125,14 +194,14 @@ __device__ __forceinline__ V* fft_lines(V* a, V* b, const FftSched& s, int ls, i
       continue;
     }
     switch (R) {
-      case 2: stage_any<V, DIR, 2>(in, out, s.L, Ns, ls, nlines, tw); break;
-      case 3: stage_any<V, DIR, 3>(in, out, s.L, Ns, ls, nlines, tw); break;
-      case 4: stage_any<V, DIR, 4>(in, out, s.L, Ns, ls, nlines, tw); break;
-      case 5: stage_any<V, DIR, 5>(in, out, s.L, Ns, ls, nlines, tw); break;
+      case 2: stage_any<V, DIR, 2>(in, out, s.L, Ns, ls, nlines, tw, sc); break;
+      case 3: stage_any<V, DIR, 3>(in, out, s.L, Ns, ls, nlines, tw, sc); break;
+      case 4: stage_any<V, DIR, 4>(in, out, s.L, Ns, ls, nlines, tw, sc); break;
+      case 5: stage_any<V, DIR, 5>(in, out, s.L, Ns, ls, nlines, tw, sc); break;
       case 16:
-        if constexpr (MR == 16) stage_any<V, DIR, 16>(in, out, s.L, Ns, ls, nlines, tw);
+        if constexpr (MR == 16) stage_any<V, DIR, 16>(in, out, s.L, Ns, ls, nlines, tw, sc);
         break;
-      default: stage_any<V, DIR, 8>(in, out, s.L, Ns, ls, nlines, tw); break;
+      default: stage_any<V, DIR, 8>(in, out, s.L, Ns, ls, nlines, tw, sc); break;
     }
     __syncthreads();
     V* t = in;
@@ -202,6 +271,25 @@ __device__ __forceinline__ void pair_offsets(const PassGeom& g, int p0, int nl, 
   }
 }
 
+// z / 2 as it goes to the spectrum (e: exponent of the line, FP64 spectrum).
+template <typename V>
+__device__ __forceinline__ V half_value(V z, int e) {
+  if constexpr (std::is_same<V, i64c>::value) return fx_pack(z, e - 1);
+  else return mk<V>(halve(z.x), halve(z.y));
+}
+// Sets the imaginary part to zero.
+template <typename V>
+__device__ __forceinline__ void drop_im(V& z) {
+  if constexpr (std::is_same<V, i64c>::value) z.y.v &= 63;   // the low bits hold the exponent
+  else z.y = typename Real<V>::T(0);
+}
+// z as it goes to the spectrum.
+template <typename V>
+__device__ __forceinline__ V spec_value(V z, int e) {
+  if constexpr (std::is_same<V, i64c>::value) return fx_pack(z, e);
+  else return z;
+}
+
 // XH: the rows are zero-padded to twice their length (free and wire BC); a
 // separate build so that the unpadded one keeps its register budget.
 template <typename V, int MR, bool XH>
@@ -215,6 +303,8 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
   const float* __restrict__ scale32 = a.in_scale32 ? a.in_scale32 + slot * b.vstride : nullptr;
   V* __restrict__ W = reinterpret_cast<V*>(a.W) + slot * a.wstride;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int scales[3][std::is_same<V, i64c>::value ? kMaxLinesPerCta : 1];
+  const LineScales sc{scales[0], scales[1], scales[2]};
   __shared__ size_t woff[2 * kMaxLinesX];
   V* tw = reinterpret_cast<V*>(smem_raw);
   const int L = s.L, ls = line_stride<V>(L);
@@ -227,6 +317,12 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
   pair_offsets<V>(g, p0, nl, woff);
   const bool red = a.red_mu && b.st;
   double sum = 0.0;
+  // FP64 spectrum: the doubles are packed as they go to shared memory
+  using I = typename std::conditional<std::is_same<V, i64c>::value, double, T>::type;
+  auto load = [&](size_t o) {
+    if constexpr (std::is_same<V, i64c>::value) return load_scaled64(in, scale, o, red, sum);
+    else return load_scaled<V>(in, scale, o, red, sum, scale32);
+  };
   {
     constexpr int U = 4;
     // XH: the padded half (j >= nx = L/2) is never read -- the first stage
@@ -234,20 +330,20 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
     // positions are staged
     LineIter it(XH ? g.nx : L);
     while (it.l < nl) {
-      T va[U], vb[U];
+      I va[U], vb[U];
       int dst[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        va[u] = T(0);
-        vb[u] = T(0);
+        va[u] = I(0);
+        vb[u] = I(0);
         dst[u] = -1;
         if (it.l < nl) {
           const int l = it.l, j = it.j;
           const int ra = 2 * (p0 + l);
           if (j < g.nx) {
             const size_t oa = (size_t)ra * g.nx + j;
-            va[u] = load_scaled<V>(in, scale, oa, red, sum, scale32);
-            if (ra + 1 < g.nrows) vb[u] = load_scaled<V>(in, scale, oa + g.nx, red, sum, scale32);
+            va[u] = load(oa);
+            if (ra + 1 < g.nrows) vb[u] = load(oa + g.nx);
           }
           dst[u] = l * ls + pidx<V>(j);
           it.next();
@@ -255,20 +351,31 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (dst[u] >= 0) b0[dst[u]] = mk<V>(va[u], vb[u]);
+        if (dst[u] >= 0) {
+          if constexpr (std::is_same<V, i64c>::value) {
+            long long re, im;
+            int e;
+            fx_of_doubles(va[u], vb[u], re, im, e);
+            b0[dst[u]] = fx_pack_normalized(re, im, e);
+          } else {
+            b0[dst[u]] = mk<V>(va[u], vb[u]);
+          }
+        }
     }
   }
   __syncthreads();
-  const V* res = fft_lines<V, -1, MR, XH>(b0, b1, s, ls, nl, tw, g.nx);
-  const T half = T(0.5);
+  if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, g.nx, 1, sc);
+  const V* res = fft_lines<V, -1, MR, XH>(b0, b1, s, ls, nl, tw, g.nx, sc);
   for (LineIter it(g.Hx); it.l < nl; it.next()) {
     const int l = it.l, k = it.j;
     const V* line = res + l * ls;
     const V zk = line[pidx<V>(k)];
     const V zm = line[pidx<V>(k == 0 ? 0 : L - k)];
     // A_k = (Z_k + conj Z_(L-k))/2 ; B_k = -i (Z_k - conj Z_(L-k))/2
-    W[woff[2 * l] + k] = mk<V>(half * (zk.x + zm.x), half * (zk.y - zm.y));
-    if (2 * (p0 + l) + 1 < g.nrows) W[woff[2 * l + 1] + k] = mk<V>(half * (zk.y + zm.y), half * (zm.x - zk.x));
+    const int e = std::is_same<V, i64c>::value ? sc.exp[l] : 0;
+    W[woff[2 * l] + k] = half_value<V>(mk<V>(zk.x + zm.x, zk.y - zm.y), e);
+    if (2 * (p0 + l) + 1 < g.nrows)
+      W[woff[2 * l + 1] + k] = half_value<V>(mk<V>(zk.y + zm.y, zm.x - zk.x), e);
   }
   if (red)
     grid_reduce(sum, b.partials + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_MU], &b.st[slot].mu_sum);
@@ -281,6 +388,8 @@ __global__ void __launch_bounds__(kThreads) k_y(PassGeom g, FftSched s, const V*
   if (slot < 0) return;
   V* __restrict__ W = reinterpret_cast<V*>(a.W) + slot * a.wstride;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int scales[3][std::is_same<V, i64c>::value ? kMaxLinesPerCta : 1];
+  const LineScales sc{scales[0], scales[1], scales[2]};
   V* tw = reinterpret_cast<V*>(smem_raw);
   const int L = s.L, ls = line_stride<V>(L), tile = g.tile_y;
   V* b0 = tw + L;
@@ -297,11 +406,13 @@ __global__ void __launch_bounds__(kThreads) k_y(PassGeom g, FftSched s, const V*
   V* col = W + plane + kx0 + c;
   if (act) load_column<V>(b0 + c * ls, col, g.Hp, y0, ystep, L, nload);
   __syncthreads();
-  const V* res = fft_lines<V, DIR, MR>(b0, b1, s, ls, nl, tw, nload);
+  if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, nload, 0, sc);
+  const V* res = fft_lines<V, DIR, MR>(b0, b1, s, ls, nl, tw, nload, sc);
   const int nstore = DIR < 0 ? L : g.ny;  // inverse: crop to y < ny
   if (act) {
     const V* line = res + c * ls;
-    for (int y = y0; y < nstore; y += ystep) col[(size_t)y * g.Hp] = line[pidx<V>(y)];
+    const int e = std::is_same<V, i64c>::value ? sc.exp[c] : 0;
+    for (int y = y0; y < nstore; y += ystep) col[(size_t)y * g.Hp] = spec_value(line[pidx<V>(y)], e);
   }
 }
 
@@ -317,6 +428,8 @@ __global__ void __launch_bounds__(kThreads) k_z(PassGeom g, FftSched s, const V*
   const bool use_k0 = a.slot_k0 && b.st && b.st[slot].use_k0;
   const double k0 = use_k0 ? b.st[slot].k0 : 0.0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int scales[3][std::is_same<V, i64c>::value ? kMaxLinesPerCta : 1];
+  const LineScales sc{scales[0], scales[1], scales[2]};
   V* tw = reinterpret_cast<V*>(smem_raw);
   const int L = s.L, ls = line_stride<V>(L), tile = g.tile_z;
   V* b0 = tw + L;
@@ -333,7 +446,8 @@ __global__ void __launch_bounds__(kThreads) k_z(PassGeom g, FftSched s, const V*
   V* col = W + colbase + c;
   if (act) load_column<V>(b0 + c * ls, col, zstride, z0, zstep, L, g.nz);
   __syncthreads();
-  V* res = fft_lines<V, -1, MR, ZH>(b0, b1, s, ls, nl, tw, g.nz);
+  if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, g.nz, 0, sc);
+  V* res = fft_lines<V, -1, MR, ZH>(b0, b1, s, ls, nl, tw, g.nz, sc);
   V* other = (res == b0) ? b1 : b0;
   const int kyp = min(ky, g.Py - ky);
   const int hy = g.Py / 2 + 1;
@@ -343,9 +457,11 @@ __global__ void __launch_bounds__(kThreads) k_z(PassGeom g, FftSched s, const V*
     const size_t tz = (size_t)hy * g.Hx;
     V* line = res + c * ls;
     const bool at0 = use_k0 && kx == 0 && ky == 0;
+    using TT = typename std::conditional<std::is_same<V, i64c>::value, double, T>::type;
+    const int e = std::is_same<V, i64c>::value ? sc.exp[c] : 0;
     constexpr int U = 8;
     for (int kb = z0; kb < L; kb += U * zstep) {
-      T t[U];
+      TT t[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int kz = min(kb + u * zstep, L - 1);
@@ -374,16 +490,25 @@ __global__ void __launch_bounds__(kThreads) k_z(PassGeom g, FftSched s, const V*
         const int kz = kb + u * zstep;
         if (kz < L) {
           const int pk = pidx<V>(kz);
-          line[pk] = cscale(line[pk], t[u]);
+          if constexpr (std::is_same<V, i64c>::value) {
+            i64c z = line[pk];
+            int ez = e;
+            fx_apply(z, ez, t[u]);
+            line[pk] = fx_pack_normalized(z.x.v, z.y.v, ez);
+          } else {
+            line[pk] = cscale(line[pk], t[u]);
+          }
         }
       }
     }
   }
   __syncthreads();
-  const V* fin = fft_lines<V, +1, MR, false>(res, other, s, ls, nl, tw, L);
+  if constexpr (std::is_same<V, i64c>::value) line_scales(res, L, ls, nl, L, 0, sc);
+  const V* fin = fft_lines<V, +1, MR, false>(res, other, s, ls, nl, tw, L, sc);
   if (act) {
     const V* line = fin + c * ls;
-    for (int z = z0; z < g.nz; z += zstep) col[(size_t)z * zstride] = line[pidx<V>(z)];
+    const int e = std::is_same<V, i64c>::value ? sc.exp[c] : 0;
+    for (int z = z0; z < g.nz; z += zstep) col[(size_t)z * zstride] = spec_value(line[pidx<V>(z)], e);
   }
 }
 
@@ -399,6 +524,8 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
   const float* __restrict__ out_scale32 = a.out_scale32 ? a.out_scale32 + slot * b.vstride : nullptr;
   const double* __restrict__ dot_with = a.dot_with ? a.dot_with + slot * b.vstride : nullptr;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int scales[3][std::is_same<V, i64c>::value ? kMaxLinesPerCta : 1];
+  const LineScales sc{scales[0], scales[1], scales[2]};
   __shared__ size_t woff[2 * kMaxLinesX];
   V* tw = reinterpret_cast<V*>(smem_raw);
   const int L = s.L, ls = line_stride<V>(L);
@@ -431,7 +558,7 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
           const V* wb = W + woff[2 * l + 1];
           A[u] = wa[k];
           if (hasb) B[u] = wb[k];
-          if (k == 0 || 2 * k == L) { A[u].y = T(0); B[u].y = T(0); }   // DC and Nyquist are real
+          if (k == 0 || 2 * k == L) { drop_im(A[u]); drop_im(B[u]); }   // DC and Nyquist are real
           dst[u] = l * ls + pidx<V>(k);
           if (k > 0 && 2 * k < L) dstm[u] = l * ls + pidx<V>(L - k);
           it.next();
@@ -440,13 +567,18 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (dst[u] >= 0) {
-          b0[dst[u]] = mk<V>(A[u].x - B[u].y, A[u].y + B[u].x);             // Z = A + i B
-          if (dstm[u] >= 0) b0[dstm[u]] = mk<V>(A[u].x + B[u].y, B[u].x - A[u].y);   // conj A + i conj B
+          int e = 0;
+          if constexpr (std::is_same<V, i64c>::value) fx_align(A[u], B[u], e);
+          const V z = mk<V>(A[u].x - B[u].y, A[u].y + B[u].x);                   // Z = A + i B
+          const V zm = mk<V>(A[u].x + B[u].y, B[u].x - A[u].y);                  // conj A + i conj B
+          b0[dst[u]] = spec_value(z, e);
+          if (dstm[u] >= 0) b0[dstm[u]] = spec_value(zm, e);
         }
     }
   }
   __syncthreads();
-  const V* res = fft_lines<V, +1, MR, false>(b0, b1, s, ls, nl, tw, L);
+  if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, L, 0, sc);
+  const V* res = fft_lines<V, +1, MR, false>(b0, b1, s, ls, nl, tw, L, sc);
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
   for (LineIter it(g.nx); it.l < nl; it.next()) {
@@ -454,17 +586,22 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
     const int ra = 2 * (p0 + l);
     const V zz = res[l * ls + pidx<V>(j)];
     const size_t oa = (size_t)ra * g.nx + j;
-    const double va = out_value<V>(zz.x, out_scale, oa, out_scale32);
-    out[oa] = va;
-    if (dot_with) dot += va * dot_with[oa];
-    if (want_wsum) wsum += unscaled<V>(zz.x);
-    if (ra + 1 < g.nrows) {
-      const size_t ob = oa + g.nx;
-      const double vb = out_value<V>(zz.y, out_scale, ob, out_scale32);
-      out[ob] = vb;
-      if (dot_with) dot += vb * dot_with[ob];
-      if (want_wsum) wsum += unscaled<V>(zz.y);
-    }
+    const int e = std::is_same<V, i64c>::value ? sc.exp[l] : 0;
+    auto store = [&](T z, size_t o) {
+      double v;
+      if constexpr (std::is_same<V, i64c>::value) {
+        const double w = unscaled<V>(z, e);
+        if (want_wsum) wsum += w;
+        v = out_scale ? w * out_scale[o] : w;
+      } else {
+        v = out_value<V>(z, out_scale, o, out_scale32);
+        if (want_wsum) wsum += unscaled<V>(z);
+      }
+      out[o] = v;
+      if (dot_with) dot += v * dot_with[o];
+    };
+    store(zz.x, oa);
+    if (ra + 1 < g.nrows) store(zz.y, oa + g.nx);
   }
   if (dot_with && b.st)
     if (grid_reduce(dot, b.partials + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_VR],
@@ -479,7 +616,7 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
 // Launchers.
 
 size_t x_lines_smem_bytes(int L, int lines, size_t vbytes) {
-  const int ls = vbytes == sizeof(double2) ? line_stride<double2>(L) : line_stride<float2>(L);
+  const int ls = vbytes == sizeof(i64c) ? line_stride<i64c>(L) : line_stride<float2>(L);
   return (size_t)(L + 2 * lines * ls) * vbytes;
 }
 
@@ -511,7 +648,7 @@ static void set_smem(K kernel, size_t bytes) {
 // Whether the schedule takes the radix-16 build of a kernel (FP64 only).
 template <typename V>
 static bool radix16(const FftSched& s) {
-  if constexpr (!std::is_same<V, double2>::value) {
+  if constexpr (!std::is_same<V, i64c>::value) {
     return false;
   } else {
     for (int k = 0; k < s.nst; ++k)
@@ -533,12 +670,26 @@ static void x_fwd_mr(const PassGeom& g, const FftSched& s, const V* tw, const Ba
   }
 }
 
+// The register-resident kernels, where they serve the length.
+template <typename V>
+static bool launch_x_reg(bool inverse, int L, const PassGeom& g, const V* tw, const Batch& b, const PipeArgs& a,
+                         int nslots, cudaStream_t st) {
+  if constexpr (std::is_same<V, i64c>::value) return launch_fix_x(inverse, L, g, tw, b, a, nslots, st);
+  else return launch_xr_pass<V>(inverse, L, g, tw, b, a, nslots, st);
+}
+template <typename V>
+static bool launch_col_reg(int mode, int L, const PassGeom& g, const V* tw, const Batch& b, const PipeArgs& a,
+                           int nslots, cudaStream_t st) {
+  if constexpr (std::is_same<V, i64c>::value) return launch_fix_col(mode, L, g, tw, b, a, nslots, st);
+  else return launch_col_pass<V>(mode, L, g, tw, b, a, nslots, st);
+}
+
 template <typename V>
 void launch_x_fwd(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
                   const PipeArgs& a, int nslots, cudaStream_t st) {
-  if (launch_xr_pass<V>(false, s.L, g, tw, b, a, nslots, st)) return;
+  if (launch_x_reg<V>(false, s.L, g, tw, b, a, nslots, st)) return;
   const size_t sm = x_lines_smem_bytes(s.L, g.lines_x, sizeof(V));
-  if constexpr (std::is_same<V, double2>::value)
+  if constexpr (std::is_same<V, i64c>::value)
     if (radix16<V>(s)) return x_fwd_mr<V, 16>(g, s, tw, b, a, nslots, sm, st);
   x_fwd_mr<V, 8>(g, s, tw, b, a, nslots, sm, st);
 }
@@ -546,11 +697,11 @@ void launch_x_fwd(const PassGeom& g, const FftSched& s, const V* tw, const Batch
 template <typename V>
 void launch_y(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
               const PipeArgs& a, bool inverse, int nslots, cudaStream_t st) {
-  if (launch_col_pass<V>(inverse ? 1 : 0, s.L, g, tw, b, a, nslots, st)) return;
+  if (launch_col_reg<V>(inverse ? 1 : 0, s.L, g, tw, b, a, nslots, st)) return;
   dim3 grid((g.Hx + g.tile_y - 1) / g.tile_y, g.nz, nslots);
   const size_t sm = x_lines_smem_bytes(s.L, g.tile_y, sizeof(V));
   count_launch();
-  if constexpr (std::is_same<V, double2>::value) {
+  if constexpr (std::is_same<V, i64c>::value) {
     if (radix16<V>(s)) {
       if (inverse) {
         set_smem(k_y<V, +1, 16>, sm);
@@ -574,12 +725,12 @@ void launch_y(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
 template <typename V>
 void launch_z(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
               const PipeArgs& a, int nslots, cudaStream_t st) {
-  if (launch_col_pass<V>(2, s.L, g, tw, b, a, nslots, st)) return;
+  if (launch_col_reg<V>(2, s.L, g, tw, b, a, nslots, st)) return;
   dim3 grid((g.Hx + g.tile_z - 1) / g.tile_z, g.Py, nslots);
   const size_t sm = x_lines_smem_bytes(s.L, g.tile_z, sizeof(V));
   count_launch();
   const bool zh = 2 * g.nz == s.L;
-  if constexpr (std::is_same<V, double2>::value) {
+  if constexpr (std::is_same<V, i64c>::value) {
     if (radix16<V>(s)) {
       if (zh) {
         set_smem(k_z<V, 16, true>, sm);
@@ -603,10 +754,10 @@ void launch_z(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
 template <typename V>
 void launch_x_inv(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
                   const PipeArgs& a, int nslots, cudaStream_t st) {
-  if (launch_xr_pass<V>(true, s.L, g, tw, b, a, nslots, st)) return;
+  if (launch_x_reg<V>(true, s.L, g, tw, b, a, nslots, st)) return;
   const size_t sm = x_lines_smem_bytes(s.L, g.lines_x, sizeof(V));
   count_launch();
-  if constexpr (std::is_same<V, double2>::value) {
+  if constexpr (std::is_same<V, i64c>::value) {
     if (radix16<V>(s)) {
       set_smem(k_x_inv<V, 16>, sm);
       k_x_inv<V, 16><<<dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st>>>(g, s, tw, b, a);
@@ -627,7 +778,7 @@ void launch_x_inv(const PassGeom& g, const FftSched& s, const V* tw, const Batch
   template void launch_x_inv<V>(const PassGeom&, const FftSched&, const V*, const Batch&,       \
                                 const PipeArgs&, int, cudaStream_t);
 
-GPS_INSTANTIATE(double2)
+GPS_INSTANTIATE(i64c)
 GPS_INSTANTIATE(float2)
 GPS_INSTANTIATE(dfc)
 

@@ -5,14 +5,49 @@
 #include <type_traits>
 
 #include "device_util.cuh"
+#include "fix64.cuh"
 #include "gps_internal.h"
 
 namespace gps {
+
+template <> struct Real<i64c> { using T = fx; };
+// Complex products of the FP64 spectrum; the factor b is in Q62 digits.
+template <> __device__ __forceinline__ i64c cmul<i64c>(i64c a, i64c b) {
+  const int dh = hi32(b.y.v), dl = lo32(b.y.v);
+  return fx_cmul(a, hi32(b.x.v), lo32(b.x.v), dh, dl, -dh, -dl);
+}
+template <> __device__ __forceinline__ i64c cmulc<i64c>(i64c a, i64c b) {
+  const int dh = hi32(b.y.v), dl = lo32(b.y.v);
+  return fx_cmul(a, hi32(b.x.v), lo32(b.x.v), -dh, -dl, dh, dl);
+}
 
 // Radix-R butterflies, DIR = -1 forward (e^{-2 pi i/R}), +1 inverse.
 template <typename V, int DIR>
 __device__ __forceinline__ V rot_i(V a) {  // a * (DIR * i)
   return DIR < 0 ? mk<V>(a.y, -a.x) : mk<V>(-a.y, a.x);
+}
+
+// k x for a constant k; x / 2; a (c + i DIR s) for constants c, s.
+template <class K, typename T>
+__device__ __forceinline__ T mulk(T x) {
+  if constexpr (std::is_same<T, fx>::value) return fx_mul(x, K::h, K::l);
+  else return T(K::d) * x;
+}
+template <typename T>
+__device__ __forceinline__ T halve(T x) {
+  if constexpr (std::is_same<T, fx>::value) return fx((x.v + 1) >> 1);
+  else return T(0.5) * x;
+}
+template <typename V, int DIR, class C, class S>
+__device__ __forceinline__ V rotk(V a) {
+  if constexpr (std::is_same<V, i64c>::value) {
+    return DIR < 0 ? fx_cmul(a, C::h, C::l, -S::h, -S::l, S::h, S::l)
+                   : fx_cmul(a, C::h, C::l, S::h, S::l, -S::h, -S::l);
+  } else {
+    using T = typename Real<V>::T;
+    const T cr = T(C::d), si = T(DIR < 0 ? -S::d : S::d);
+    return mk<V>(a.x * cr - a.y * si, a.x * si + a.y * cr);
+  }
 }
 
 template <typename V, int DIR, int R> struct Dft;
@@ -50,21 +85,19 @@ template <typename V, int DIR> struct Dft<V, DIR, 4> {
 
 template <typename V, int DIR> struct Dft<V, DIR, 8> {
   __device__ __forceinline__ static void run(V* x) {
-    using T = typename Real<V>::T;
-    const T c = (T)0.70710678118654752440;  // sqrt(1/2)
     V e[4] = {x[0], x[2], x[4], x[6]};
     V o[4] = {x[1], x[3], x[5], x[7]};
     Dft<V, DIR, 4>::run(e);
     Dft<V, DIR, 4>::run(o);
     // o_k *= e^{DIR 2 pi i k / 8}
     if (DIR < 0) {
-      o[1] = mk<V>(c * (o[1].x + o[1].y), c * (o[1].y - o[1].x));
+      o[1] = mk<V>(mulk<KSqrtHalf>(o[1].x + o[1].y), mulk<KSqrtHalf>(o[1].y - o[1].x));
       o[2] = mk<V>(o[2].y, -o[2].x);
-      o[3] = mk<V>(c * (o[3].y - o[3].x), -c * (o[3].x + o[3].y));
+      o[3] = mk<V>(mulk<KSqrtHalf>(o[3].y - o[3].x), mulk<KNeg<KSqrtHalf>>(o[3].x + o[3].y));
     } else {
-      o[1] = mk<V>(c * (o[1].x - o[1].y), c * (o[1].x + o[1].y));
+      o[1] = mk<V>(mulk<KSqrtHalf>(o[1].x - o[1].y), mulk<KSqrtHalf>(o[1].x + o[1].y));
       o[2] = mk<V>(-o[2].y, o[2].x);
-      o[3] = mk<V>(-c * (o[3].x + o[3].y), c * (o[3].x - o[3].y));
+      o[3] = mk<V>(mulk<KNeg<KSqrtHalf>>(o[3].x + o[3].y), mulk<KSqrtHalf>(o[3].x - o[3].y));
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -73,19 +106,17 @@ template <typename V, int DIR> struct Dft<V, DIR, 8> {
     }
   }
   __device__ __forceinline__ static void run_half(V* x) {
-    using T = typename Real<V>::T;
-    const T c = (T)0.70710678118654752440;  // sqrt(1/2)
     V e[4] = {x[0], x[1], x[2], x[3]};
     V o[4] = {x[0], x[1], x[2], x[3]};
     // o_r *= e^{DIR 2 pi i r / 8}
     if (DIR < 0) {
-      o[1] = mk<V>(c * (o[1].x + o[1].y), c * (o[1].y - o[1].x));
+      o[1] = mk<V>(mulk<KSqrtHalf>(o[1].x + o[1].y), mulk<KSqrtHalf>(o[1].y - o[1].x));
       o[2] = mk<V>(o[2].y, -o[2].x);
-      o[3] = mk<V>(c * (o[3].y - o[3].x), -c * (o[3].x + o[3].y));
+      o[3] = mk<V>(mulk<KSqrtHalf>(o[3].y - o[3].x), mulk<KNeg<KSqrtHalf>>(o[3].x + o[3].y));
     } else {
-      o[1] = mk<V>(c * (o[1].x - o[1].y), c * (o[1].x + o[1].y));
+      o[1] = mk<V>(mulk<KSqrtHalf>(o[1].x - o[1].y), mulk<KSqrtHalf>(o[1].x + o[1].y));
       o[2] = mk<V>(-o[2].y, o[2].x);
-      o[3] = mk<V>(-c * (o[3].x + o[3].y), c * (o[3].x - o[3].y));
+      o[3] = mk<V>(mulk<KNeg<KSqrtHalf>>(o[3].x + o[3].y), mulk<KSqrtHalf>(o[3].x - o[3].y));
     }
     Dft<V, DIR, 4>::run(e);
     Dft<V, DIR, 4>::run(o);
@@ -100,17 +131,7 @@ template <typename V, int DIR> struct Dft<V, DIR, 8> {
 // 16 points as two 8-point transforms of the even and odd elements joined by
 // the twiddles e^{DIR 2 pi i k / 16}, k = 0..7.
 template <typename V, int DIR> struct Dft<V, DIR, 16> {
-  __device__ __forceinline__ static V rot(V a, typename Real<V>::T cr, typename Real<V>::T sr) {
-    // a (cr + i DIR sr)
-    using T = typename Real<V>::T;
-    const T si = DIR < 0 ? -sr : sr;
-    return mk<V>(a.x * cr - a.y * si, a.x * si + a.y * cr);
-  }
   __device__ __forceinline__ static void run(V* x) {
-    using T = typename Real<V>::T;
-    const T c1 = (T)0.92387953251128675613;   // cos(pi/8)
-    const T s1 = (T)0.38268343236508977173;   // sin(pi/8)
-    const T c = (T)0.70710678118654752440;    // sqrt(1/2)
     V e[8], o[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -119,13 +140,13 @@ template <typename V, int DIR> struct Dft<V, DIR, 16> {
     }
     Dft<V, DIR, 8>::run(e);
     Dft<V, DIR, 8>::run(o);
-    o[1] = rot(o[1], c1, s1);
-    o[2] = rot(o[2], c, c);
-    o[3] = rot(o[3], s1, c1);
+    o[1] = rotk<V, DIR, KCosPi8, KSinPi8>(o[1]);
+    o[2] = rotk<V, DIR, KSqrtHalf, KSqrtHalf>(o[2]);
+    o[3] = rotk<V, DIR, KSinPi8, KCosPi8>(o[3]);
     o[4] = DIR < 0 ? mk<V>(o[4].y, -o[4].x) : mk<V>(-o[4].y, o[4].x);
-    o[5] = rot(o[5], -s1, c1);
-    o[6] = rot(o[6], -c, c);
-    o[7] = rot(o[7], -c1, s1);
+    o[5] = rotk<V, DIR, KNeg<KSinPi8>, KCosPi8>(o[5]);
+    o[6] = rotk<V, DIR, KNeg<KSqrtHalf>, KSqrtHalf>(o[6]);
+    o[7] = rotk<V, DIR, KNeg<KCosPi8>, KSinPi8>(o[7]);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       x[k] = cadd(e[k], o[k]);
@@ -133,21 +154,17 @@ template <typename V, int DIR> struct Dft<V, DIR, 16> {
     }
   }
   __device__ __forceinline__ static void run_half(V* x) {
-    using T = typename Real<V>::T;
-    const T c1 = (T)0.92387953251128675613;   // cos(pi/8)
-    const T s1 = (T)0.38268343236508977173;   // sin(pi/8)
-    const T c = (T)0.70710678118654752440;    // sqrt(1/2)
     V e[8], o[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) e[r] = x[r];
     o[0] = x[0];
-    o[1] = rot(x[1], c1, s1);
-    o[2] = rot(x[2], c, c);
-    o[3] = rot(x[3], s1, c1);
+    o[1] = rotk<V, DIR, KCosPi8, KSinPi8>(x[1]);
+    o[2] = rotk<V, DIR, KSqrtHalf, KSqrtHalf>(x[2]);
+    o[3] = rotk<V, DIR, KSinPi8, KCosPi8>(x[3]);
     o[4] = DIR < 0 ? mk<V>(x[4].y, -x[4].x) : mk<V>(-x[4].y, x[4].x);
-    o[5] = rot(x[5], -s1, c1);
-    o[6] = rot(x[6], -c, c);
-    o[7] = rot(x[7], -c1, s1);
+    o[5] = rotk<V, DIR, KNeg<KSinPi8>, KCosPi8>(x[5]);
+    o[6] = rotk<V, DIR, KNeg<KSqrtHalf>, KSqrtHalf>(x[6]);
+    o[7] = rotk<V, DIR, KNeg<KCosPi8>, KSinPi8>(x[7]);
     Dft<V, DIR, 8>::run(e);
     Dft<V, DIR, 8>::run(o);
 #pragma unroll
@@ -160,12 +177,11 @@ template <typename V, int DIR> struct Dft<V, DIR, 16> {
 
 template <typename V, int DIR> struct Dft<V, DIR, 3> {
   __device__ __forceinline__ static void run(V* x) {
-    using T = typename Real<V>::T;
-    const T s3 = (T)0.86602540378443864676;  // sqrt(3)/2
+    using s3 = typename std::conditional<(DIR > 0), KSqrt3Half, KNeg<KSqrt3Half>>::type;
     V t1 = cadd(x[1], x[2]);
-    V t2 = mk<V>(x[0].x - (T)0.5 * t1.x, x[0].y - (T)0.5 * t1.y);
+    V t2 = mk<V>(x[0].x - halve(t1.x), x[0].y - halve(t1.y));
     V d = csub(x[1], x[2]);
-    V u = mk<V>((T)DIR * s3 * d.x, (T)DIR * s3 * d.y);   // u = DIR s3 (x1 - x2)
+    V u = mk<V>(mulk<s3>(d.x), mulk<s3>(d.y));   // u = DIR sqrt(3)/2 (x1 - x2)
     V iu = mk<V>(-u.y, u.x);
     x[0] = cadd(x[0], t1);
     x[1] = cadd(t2, iu);
@@ -175,17 +191,16 @@ template <typename V, int DIR> struct Dft<V, DIR, 3> {
 
 template <typename V, int DIR> struct Dft<V, DIR, 5> {
   __device__ __forceinline__ static void run(V* x) {
-    using T = typename Real<V>::T;
-    const T c1 = (T)0.30901699437494742410;   // cos(2 pi/5) = (sqrt5 - 1)/4
-    const T c2 = (T)-0.80901699437494742410;  // cos(4 pi/5) = -(sqrt5 + 1)/4
-    const T s1 = (T)0.95105651629515357212;   // sin(2 pi/5)
-    const T s2 = (T)0.58778525229247312917;   // sin(4 pi/5)
+    using c1 = KCos2Pi5;
+    using c2 = KCos4Pi5;
+    using s1 = typename std::conditional<(DIR > 0), KSin2Pi5, KNeg<KSin2Pi5>>::type;
+    using s2 = typename std::conditional<(DIR > 0), KSin4Pi5, KNeg<KSin4Pi5>>::type;
     V a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]);
     V a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
-    V p1 = mk<V>(x[0].x + c1 * a1.x + c2 * a2.x, x[0].y + c1 * a1.y + c2 * a2.y);
-    V p2 = mk<V>(x[0].x + c2 * a1.x + c1 * a2.x, x[0].y + c2 * a1.y + c1 * a2.y);
-    V q1 = mk<V>((T)DIR * (s1 * b1.x + s2 * b2.x), (T)DIR * (s1 * b1.y + s2 * b2.y));
-    V q2 = mk<V>((T)DIR * (s2 * b1.x - s1 * b2.x), (T)DIR * (s2 * b1.y - s1 * b2.y));
+    V p1 = mk<V>(x[0].x + mulk<c1>(a1.x) + mulk<c2>(a2.x), x[0].y + mulk<c1>(a1.y) + mulk<c2>(a2.y));
+    V p2 = mk<V>(x[0].x + mulk<c2>(a1.x) + mulk<c1>(a2.x), x[0].y + mulk<c2>(a1.y) + mulk<c1>(a2.y));
+    V q1 = mk<V>(mulk<s1>(b1.x) + mulk<s2>(b2.x), mulk<s1>(b1.y) + mulk<s2>(b2.y));
+    V q2 = mk<V>(mulk<s2>(b1.x) - mulk<s1>(b2.x), mulk<s2>(b1.y) - mulk<s1>(b2.y));
     V iq1 = mk<V>(-q1.y, q1.x), iq2 = mk<V>(-q2.y, q2.x);
     x[0] = cadd(x[0], cadd(a1, a2));
     x[1] = cadd(p1, iq1);
@@ -196,15 +211,15 @@ template <typename V, int DIR> struct Dft<V, DIR, 5> {
 };
 
 // Shared-memory layout of a line: one pad element after every 128 bytes
-// (8 complex doubles, 16 complex floats), so that the stride-R scatters of
+// (8 complex values of 16 bytes, 16 complex floats), so that the stride-R scatters of
 // the early Stockham stages spread over all banks.
 template <typename V> struct PadShift;
-template <> struct PadShift<double2> { static constexpr int v = 3; };
 template <> struct PadShift<float2> { static constexpr int v = 4; };
 template <> struct PadShift<dfc> { static constexpr int v = 3; };
+template <> struct PadShift<i64c> { static constexpr int v = 3; };
 
 template <typename V> struct SpecOf;
-template <> struct SpecOf<double2> { static constexpr int v = SPEC_FP64; };
+template <> struct SpecOf<i64c> { static constexpr int v = SPEC_FP64; };
 template <> struct SpecOf<float2> { static constexpr int v = SPEC_FP32; };
 template <> struct SpecOf<dfc> { static constexpr int v = SPEC_DF64; };
 
@@ -236,35 +251,41 @@ __device__ __forceinline__ int pass_slot(const Batch& b) {
   return s;
 }
 
-// Input value of the x pass: in * scale, rounded to the spectrum's real type.
-// The FP32 spectrum multiplies in FP32 unless the FP64 sum of the products is
-// wanted; conversions run on the integer pipe.
+// Input value of the x pass, in * scale: the FP64 product ...
+__device__ __forceinline__ double load_scaled64(const double* in, const double* scale, size_t o, bool red,
+                                                double& sum) {
+  double v = in[o];
+  if (scale) v *= scale[o];
+  if (red) sum += v;
+  return v;
+}
+// ... rounded to the spectrum's real type.  The FP32 spectrum multiplies in
+// FP32 unless the FP64 sum of the products is wanted; conversions run on the
+// integer pipe.
 template <typename V>
 __device__ __forceinline__ typename Real<V>::T load_scaled(const double* in, const double* scale,
                                                            size_t o, bool red, double& sum,
                                                            const float* scale32 = nullptr) {
   if constexpr (std::is_same<V, float2>::value) {
-    if (red) {
-      double v = in[o];
-      if (scale) v *= scale[o];
-      sum += v;
-      return d2f_rn(v);
-    }
+    if (red) return d2f_rn(load_scaled64(in, scale, o, red, sum));
     float v = d2f_rn(in[o]);
     if (scale32) v *= scale32[o];
     else if (scale) v *= d2f_rn(scale[o]);
     return v;
   } else {
-    double v = in[o];
-    if (scale) v *= scale[o];
-    if (red) sum += v;
-    if constexpr (std::is_same<V, dfc>::value) return df_of(v);
-    else return v;
+    return df_of(load_scaled64(in, scale, o, red, sum));
   }
 }
 
 // Real output value of the x inverse pass as a double (integer-pipe
-// conversions; the FP32 spectrum scales in FP32).
+// conversions; the FP32 spectrum scales in FP32).  e: exponent of the line
+// (FP64 spectrum only).
+template <typename V>
+__device__ __forceinline__ double unscaled(typename Real<V>::T z, int e = 0) {
+  if constexpr (std::is_same<V, float2>::value) return f2d(z);
+  else if constexpr (std::is_same<V, dfc>::value) return dbl_of(z);
+  else return fx_to_double(z.v, e);
+}
 template <typename V>
 __device__ __forceinline__ double out_value(typename Real<V>::T z, const double* scale, size_t o,
                                             const float* scale32 = nullptr) {
@@ -274,19 +295,10 @@ __device__ __forceinline__ double out_value(typename Real<V>::T z, const double*
     else if (scale) v *= d2f_rn(scale[o]);
     return f2d(v);
   } else {
-    double v;
-    if constexpr (std::is_same<V, dfc>::value) v = dbl_of(z);
-    else v = z;
+    double v = unscaled<V>(z);
     if (scale) v *= scale[o];
     return v;
   }
-}
-
-template <typename V>
-__device__ __forceinline__ double unscaled(typename Real<V>::T z) {
-  if constexpr (std::is_same<V, float2>::value) return f2d(z);
-  else if constexpr (std::is_same<V, dfc>::value) return dbl_of(z);
-  else return z;
 }
 
 }  // namespace gps

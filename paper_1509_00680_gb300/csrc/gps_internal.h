@@ -114,6 +114,7 @@ struct PassGeom {
   int tile_y, tile_z;  // columns per CTA in the y / z passes
   int x_reg;           // FP32 spectrum: 1 = x passes by the register-resident kernels
   int z_tma;           // FP32 / df64 spectrum: 1 = z pass by the TMA-staged kernel
+  int plain_tw;        // FP64 spectrum: 1 = only the plain twiddle table exists (no per-stage layouts)
 };
 
 // Slot addressing of one launch.  active == nullptr: slot 0 only, no phase
@@ -178,11 +179,17 @@ template <typename V>
 void launch_x_inv(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
                   const PipeArgs& a, int nslots, cudaStream_t st);
 // Register-resident column passes (fft_col.cu) for power-of-two lengths
-// 64 .. 1024: mode 0 y forward, 1 y inverse, 2 z.  false: length not covered
-// (and always for the FP64 spectrum).  Their twiddle array `tw` must hold
+// 64 .. 1024: mode 0 y forward, 1 y inverse, 2 z.  false: length not covered.
+// Their twiddle array `tw` must hold
 // 3 L entries: the plain table and the two per-stage layouts whose plain
 // indices col_stage_twiddle_index(L, idx[2 L]) writes (forward, reversed).
 bool col_pass_supported(int L);
+// The same for the FP64 spectrum (fft_fix.cu): row passes and column passes.
+struct i64c;
+bool launch_fix_x(bool inverse, int L, const PassGeom& g, const i64c* tw, const Batch& b, const PipeArgs& a,
+                  int nslots, cudaStream_t st);
+bool launch_fix_col(int mode, int L, const PassGeom& g, const i64c* tw, const Batch& b, const PipeArgs& a,
+                    int nslots, cudaStream_t st);
 // Bounded device waits (TMA-staged passes) that gave up since the last call;
 // resets the count.
 unsigned int take_wait_timeouts();

@@ -12,6 +12,7 @@
 // every GPU that loads this library holds it until the process exits.
 #include <mutex>
 
+#include "fix64.cuh"
 #include "gps_internal.h"
 #include "kernels.h"
 
@@ -62,12 +63,13 @@ bool radix_schedule(int L, gps::FftSched* s) {
   return rem == 1;
 }
 
-// tw[m] = exp(-2 pi i m / L) in FP64.
-__global__ void k_noalloc_twiddles(double2* tw, int L) {
+// tw[m] = exp(-2 pi i m / L), evaluated in FP64, as Q62 digits.
+__global__ void k_noalloc_twiddles(gps::i64c* tw, int L) {
   for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
     double s, c;
     sincospi(2.0 * (double)m / (double)L, &s, &c);
-    tw[m] = make_double2(c, -s);
+    tw[m].x.v = gps::q62_digits(__double2ll_rn(c * 4611686018427387904.0));
+    tw[m].y.v = gps::q62_digits(__double2ll_rn(-s * 4611686018427387904.0));
   }
 }
 
@@ -92,12 +94,12 @@ extern "C" int gps_vacuum_solve_noalloc(const gps_grid* grid, const double* sigm
   const size_t table_n = (size_t)Hx * hy * hz;
   // scratch layout: twiddles x, y, z | Green's-function table | spectrum
   const size_t off_twx = 0;
-  const size_t off_twy = off_twx + align256((size_t)Px * sizeof(double2));
-  const size_t off_twz = off_twy + align256((size_t)Py * sizeof(double2));
-  const size_t off_tab = off_twz + align256((size_t)Pz * sizeof(double2));
+  const size_t off_twy = off_twx + align256((size_t)Px * sizeof(i64c));
+  const size_t off_twz = off_twy + align256((size_t)Py * sizeof(i64c));
+  const size_t off_tab = off_twz + align256((size_t)Pz * sizeof(i64c));
   const size_t off_w = off_tab + align256(table_n * sizeof(double));
   const int Hp = spectrum_pitch(Hx);
-  const size_t need = off_w + (size_t)Hp * Py * grid->nz * sizeof(double2);
+  const size_t need = off_w + (size_t)Hp * Py * grid->nz * sizeof(i64c);
   if (need > kScratchBytes) return GPS_ERR_INVALID;   // beyond the fixed scratch size
 
   int device = 0;
@@ -106,11 +108,11 @@ extern "C" int gps_vacuum_solve_noalloc(const gps_grid* grid, const double* sigm
   int e = scratch_address(device, reinterpret_cast<void**>(&base));
   if (e != GPS_OK) return e;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double2* twx = reinterpret_cast<double2*>(base + off_twx);
-  double2* twy = reinterpret_cast<double2*>(base + off_twy);
-  double2* twz = reinterpret_cast<double2*>(base + off_twz);
+  i64c* twx = reinterpret_cast<i64c*>(base + off_twx);
+  i64c* twy = reinterpret_cast<i64c*>(base + off_twy);
+  i64c* twz = reinterpret_cast<i64c*>(base + off_twz);
   double* table = reinterpret_cast<double*>(base + off_tab);
-  double2* W = reinterpret_cast<double2*>(base + off_w);
+  i64c* W = reinterpret_cast<i64c*>(base + off_w);
 
   // Tables are rebuilt on every call: the array keeps whatever the previous
   // call (of any grid) left in it.  The spectrum needs no clearing: every
@@ -130,24 +132,25 @@ extern "C" int gps_vacuum_solve_noalloc(const gps_grid* grid, const double* sigm
   else
     launch_table_surface(table, Hx, hy, hz, dkx, dky, dkz, grid->nz * grid->hz, inv_n, st);
 
-  PassGeom g;
+  PassGeom g{};
   g.nx = grid->nx; g.ny = grid->ny; g.nz = grid->nz;
   g.Px = Px; g.Py = Py; g.Pz = Pz; g.Hx = Hx; g.Hp = Hp;
   g.nrows = grid->ny * grid->nz;
-  g.lines_x = default_lines(Px, (g.nrows + 1) / 2, sizeof(double2));
-  g.tile_y = default_lines(Py, Hx * grid->nz, sizeof(double2));
-  g.tile_z = default_lines(Pz, Hx * Py, sizeof(double2));
+  g.lines_x = default_lines(Px, (g.nrows + 1) / 2, sizeof(i64c));
+  g.tile_y = default_lines(Py, Hx * grid->nz, sizeof(i64c));
+  g.tile_z = default_lines(Pz, Hx * Py, sizeof(i64c));
+  g.plain_tw = 1;            // the scratch array holds the plain twiddle tables only
   Batch b{};                 // one slot, no phase machine
   PipeArgs a{};
   a.in = sigma_dev;
   a.out = w_dev;
   a.table = table;
   a.W = W;
-  launch_x_fwd<double2>(g, sx, twx, b, a, 1, st);
-  launch_y<double2>(g, sy, twy, b, a, false, 1, st);
-  launch_z<double2>(g, sz, twz, b, a, 1, st);
-  launch_y<double2>(g, sy, twy, b, a, true, 1, st);
-  launch_x_inv<double2>(g, sx, twx, b, a, 1, st);
+  launch_x_fwd<i64c>(g, sx, twx, b, a, 1, st);
+  launch_y<i64c>(g, sy, twy, b, a, false, 1, st);
+  launch_z<i64c>(g, sz, twz, b, a, 1, st);
+  launch_y<i64c>(g, sy, twy, b, a, true, 1, st);
+  launch_x_inv<i64c>(g, sx, twx, b, a, 1, st);
   if (cudaGetLastError() != cudaSuccess) return GPS_ERR_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return GPS_ERR_CUDA;
   return GPS_OK;
