@@ -165,22 +165,39 @@ template <> __device__ __forceinline__ dfc cmulc<dfc>(dfc a, dfc b) {
   return mk<dfc>(df_dot2<+1>(a.x, b.x, a.y, b.y), df_dot2<-1>(a.y, b.x, a.x, b.y));
 }
 
-// Sum of v over the block (any blockDim.x multiple of 32, <= 1024); result
-// valid in every thread.
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double warp_part[32];
-  __shared__ double total;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) warp_part[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    double t = lane < nw ? warp_part[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) total = t;
+// Sums of K values over the block (blockDim.x a multiple of 32, at most 256):
+// sum k ends up in the first lane of warp k.  The FP64 pipe takes 16 cycles
+// for a warp's addition, so the lanes are folded once by a shuffle and the
+// rest goes through shared memory to one warp per sum: 16 warp additions a
+// sum and 256-thread block against 45 of a shuffle tree in every warp.
+// Needs a __syncthreads() before it is called again.
+template <int K>
+__device__ __forceinline__ double block_sums(const double (&v)[K]) {
+  __shared__ double sh[K][128];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const double x = v[k] + __shfl_down_sync(0xffffffffu, v[k], 16);
+    if (lane < 16) sh[k][wid * 16 + lane] = x;
   }
+  __syncthreads();
+  double x = 0.0;
+  if (wid < K) {
+    const double* a = sh[0] + wid * 128 + lane;      // 16 nw values of sum wid
+    if (nw == 8) x = (a[0] + a[32]) + (a[64] + a[96]);
+    else
+      for (int i = lane; i < 16 * nw; i += 32) x += sh[wid][i];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+  }
+  return x;
+}
+
+// Sum of v over the block; result valid in every thread.
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double total;
+  const double a[1] = {v};
+  const double x = block_sums(a);
+  if (threadIdx.x == 0) total = x;
   __syncthreads();
   return total;
 }
@@ -189,112 +206,69 @@ __device__ __forceinline__ double block_sum(double v) {
 __device__ __forceinline__ unsigned int linear_block() { return blockIdx.x + gridDim.x * blockIdx.y; }
 __device__ __forceinline__ unsigned int num_blocks() { return gridDim.x * gridDim.y; }
 
-// Deterministic grid reduction over the blocks of one slot: every block stores
-// its partial; the last block to arrive (atomic ticket) sums all partials in
-// a fixed order and returns true in all of its threads with *result set.  The sum order does not depend
-// on which block arrives last, so results are bitwise reproducible.
-__device__ __forceinline__ bool grid_reduce(double v, double* partials, unsigned int* counter,
-                                            double* result) {
+// Deterministic grid reduction of K sums over the blocks of one slot: every
+// block stores its partials; the last block to arrive (one atomic ticket)
+// sums all partials in a fixed order and returns true in all of its threads
+// with *res[k] set.  The sum order does not depend on which block arrives
+// last, so results are bitwise reproducible.  The last block keeps eight
+// loads of each sum in flight per thread: up to 8192 partials, in a tail
+// that nothing overlaps.
+template <int K>
+__device__ __forceinline__ bool grid_reduce_k(const double (&v)[K], double* const (&part)[K], unsigned int* counter,
+                                              double* const (&res)[K]) {
+  static_assert(K <= 4, "one warp per sum");
   __shared__ bool am_last;
-  const double bs = block_sum(v);
-  if (threadIdx.x == 0) {
-    partials[linear_block()] = bs;
-    __threadfence();
-    const unsigned int t = atomicAdd(counter, 1u);
-    am_last = (t == num_blocks() - 1);
-  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();
+  const double bs = block_sums(v);
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (wid == k && lane == 0) part[k][linear_block()] = bs;
+  if (wid < K && lane == 0) __threadfence();
+  if (K > 1) __syncthreads();
+  if (threadIdx.x == 0) am_last = atomicAdd(counter, 1u) == num_blocks() - 1;
   __syncthreads();
   if (!am_last) return false;
   __threadfence();
-  const unsigned int nb = num_blocks();
-  double s = 0.0;
-  for (unsigned int i = threadIdx.x; i < nb; i += blockDim.x) s += __ldcg(partials + i);
-  s = block_sum(s);
-  if (threadIdx.x == 0) {
-    *result = s;
-    *counter = 0u;
+  const unsigned int nb = num_blocks(), bd = blockDim.x;
+  double s[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) s[k] = 0.0;
+  for (unsigned int i = threadIdx.x; i < nb; i += 8 * bd) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t[u] = i + u * bd < nb ? __ldcg(part[k] + i + u * bd) : 0.0;
+      if (i + 4 * bd < nb) s[k] += (t[4] + t[5]) + (t[6] + t[7]);
+      s[k] += (t[0] + t[1]) + (t[2] + t[3]);
+    }
   }
+  const double total = block_sums(s);
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (wid == k && lane == 0) *res[k] = total;
+  if (threadIdx.x == 0) *counter = 0u;
+  __threadfence_block();
   __syncthreads();
   return true;
 }
 
-// Three sums over the blocks of one slot in one pass (one block reduction,
-// one atomic ticket, one last-block tail); same fixed-order determinism as
-// grid_reduce.
+__device__ __forceinline__ bool grid_reduce(double v, double* partials, unsigned int* counter,
+                                            double* result) {
+  const double a[1] = {v};
+  double* const p[1] = {partials};
+  double* const r[1] = {result};
+  return grid_reduce_k(a, p, counter, r);
+}
+
 __device__ __forceinline__ bool grid_reduce3(double a, double b, double c, double* pa, double* pb,
                                              double* pc, unsigned int* counter, double* ra,
                                              double* rb, double* rc) {
-  __shared__ double part[3][32];
-  __shared__ bool am_last;
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-    c += __shfl_down_sync(0xffffffffu, c, o);
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  __syncthreads();
-  if (lane == 0) {
-    part[0][wid] = a;
-    part[1][wid] = b;
-    part[2][wid] = c;
-  }
-  __syncthreads();
-  if (wid == 0) {
-    double x = lane < nw ? part[0][lane] : 0.0;
-    double y = lane < nw ? part[1][lane] : 0.0;
-    double z = lane < nw ? part[2][lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) {
-      x += __shfl_down_sync(0xffffffffu, x, o);
-      y += __shfl_down_sync(0xffffffffu, y, o);
-      z += __shfl_down_sync(0xffffffffu, z, o);
-    }
-    if (lane == 0) {
-      const unsigned int lb = linear_block();
-      pa[lb] = x;
-      pb[lb] = y;
-      pc[lb] = z;
-      __threadfence();
-      const unsigned int t = atomicAdd(counter, 1u);
-      am_last = (t == num_blocks() - 1);
-    }
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  const unsigned int nb = num_blocks();
-  double x = 0.0, y = 0.0, z = 0.0;
-  for (unsigned int i = threadIdx.x; i < nb; i += blockDim.x) {
-    x += __ldcg(pa + i);
-    y += __ldcg(pb + i);
-    z += __ldcg(pc + i);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_down_sync(0xffffffffu, x, o);
-    y += __shfl_down_sync(0xffffffffu, y, o);
-    z += __shfl_down_sync(0xffffffffu, z, o);
-  }
-  __syncthreads();
-  if (lane == 0) {
-    part[0][wid] = x;
-    part[1][wid] = y;
-    part[2][wid] = z;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sx = 0.0, sy = 0.0, sz = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      sx += part[0][w];
-      sy += part[1][w];
-      sz += part[2][w];
-    }
-    *ra = sx;
-    *rb = sy;
-    *rc = sz;
-    *counter = 0u;
-  }
-  __syncthreads();
-  return true;
+  const double v[3] = {a, b, c};
+  double* const p[3] = {pa, pb, pc};
+  double* const r[3] = {ra, rb, rc};
+  return grid_reduce_k(v, p, counter, r);
 }
 
 }  // namespace gps

@@ -317,48 +317,96 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
   pair_offsets<V>(g, p0, nl, woff);
   const bool red = a.red_mu && b.st;
   double sum = 0.0;
-  // FP64 spectrum: the doubles are packed as they go to shared memory
-  using I = typename std::conditional<std::is_same<V, i64c>::value, double, T>::type;
-  auto load = [&](size_t o) {
-    if constexpr (std::is_same<V, i64c>::value) return load_scaled64(in, scale, o, red, sum);
-    else return load_scaled<V>(in, scale, o, red, sum, scale32);
-  };
   {
     constexpr int U = 4;
     // XH: the padded half (j >= nx = L/2) is never read -- the first stage
     // runs on the lower half only (fft_lines prunes it) -- so only the data
-    // positions are staged
+    // positions are staged.  The loads of a batch are issued before any of
+    // them is used.
     LineIter it(XH ? g.nx : L);
     while (it.l < nl) {
-      I va[U], vb[U];
+      double va[U], vb[U];
+      size_t oa[U];
       int dst[U];
+      bool ina[U], inb[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        va[u] = I(0);
-        vb[u] = I(0);
         dst[u] = -1;
+        ina[u] = false;
+        inb[u] = false;
+        oa[u] = 0;
         if (it.l < nl) {
           const int l = it.l, j = it.j;
           const int ra = 2 * (p0 + l);
-          if (j < g.nx) {
-            const size_t oa = (size_t)ra * g.nx + j;
-            va[u] = load(oa);
-            if (ra + 1 < g.nrows) vb[u] = load(oa + g.nx);
-          }
+          ina[u] = j < g.nx;
+          inb[u] = ina[u] && ra + 1 < g.nrows;
+          oa[u] = (size_t)ra * g.nx + j;
           dst[u] = l * ls + pidx<V>(j);
           it.next();
         }
       }
 #pragma unroll
+      for (int u = 0; u < U; ++u) {
+        va[u] = ina[u] ? in[oa[u]] : 0.0;
+        vb[u] = inb[u] ? in[oa[u] + g.nx] : 0.0;
+      }
+      if constexpr (std::is_same<V, float2>::value) {
+        if (!red) {
+          float fa[U], fb[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            fa[u] = d2f_rn(va[u]);
+            fb[u] = d2f_rn(vb[u]);
+          }
+          if (scale32) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              fa[u] *= ina[u] ? scale32[oa[u]] : 0.f;
+              fb[u] *= inb[u] ? scale32[oa[u] + g.nx] : 0.f;
+            }
+          } else if (scale) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              fa[u] *= ina[u] ? d2f_rn(scale[oa[u]]) : 0.f;
+              fb[u] *= inb[u] ? d2f_rn(scale[oa[u] + g.nx]) : 0.f;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (dst[u] >= 0) b0[dst[u]] = mk<V>(fa[u], fb[u]);
+          continue;
+        }
+      }
+      if (scale) {
+        double sa[U], sb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          sa[u] = ina[u] ? scale[oa[u]] : 0.0;
+          sb[u] = inb[u] ? scale[oa[u] + g.nx] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          va[u] *= sa[u];
+          vb[u] *= sb[u];
+        }
+      }
+      if (red) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) sum += va[u] + vb[u];
+      }
+#pragma unroll
       for (int u = 0; u < U; ++u)
         if (dst[u] >= 0) {
           if constexpr (std::is_same<V, i64c>::value) {
+            // FP64 spectrum: the doubles are packed as they go to shared memory
             long long re, im;
             int e;
             fx_of_doubles(va[u], vb[u], re, im, e);
             b0[dst[u]] = fx_pack_normalized(re, im, e);
+          } else if constexpr (std::is_same<V, float2>::value) {
+            b0[dst[u]] = mk<V>(d2f_rn(va[u]), d2f_rn(vb[u]));
           } else {
-            b0[dst[u]] = mk<V>(va[u], vb[u]);
+            b0[dst[u]] = mk<V>(df_of(va[u]), df_of(vb[u]));
           }
         }
     }
@@ -581,35 +629,110 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
   const V* res = fft_lines<V, +1, MR, false>(b0, b1, s, ls, nl, tw, L, sc);
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
-  for (LineIter it(g.nx); it.l < nl; it.next()) {
-    const int l = it.l, j = it.j;
-    const int ra = 2 * (p0 + l);
-    const V zz = res[l * ls + pidx<V>(j)];
-    const size_t oa = (size_t)ra * g.nx + j;
-    const int e = std::is_same<V, i64c>::value ? sc.exp[l] : 0;
-    auto store = [&](T z, size_t o) {
-      double v;
-      if constexpr (std::is_same<V, i64c>::value) {
-        const double w = unscaled<V>(z, e);
-        if (want_wsum) wsum += w;
-        v = out_scale ? w * out_scale[o] : w;
-      } else {
-        v = out_value<V>(z, out_scale, o, out_scale32);
-        if (want_wsum) wsum += unscaled<V>(z);
+  {
+    // batches whose scale factors and r are loaded before anything is stored
+    constexpr int U = 4;
+    LineIter it(g.nx);
+    while (it.l < nl) {
+      V z[U];
+      size_t oa[U];
+      int e[U];
+      bool ina[U], inb[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        ina[u] = it.l < nl;
+        inb[u] = false;
+        z[u] = czero<V>();
+        oa[u] = 0;
+        e[u] = 0;
+        if (ina[u]) {
+          const int l = it.l, j = it.j;
+          const int ra = 2 * (p0 + l);
+          inb[u] = ra + 1 < g.nrows;
+          oa[u] = (size_t)ra * g.nx + j;
+          z[u] = res[l * ls + pidx<V>(j)];
+          if constexpr (std::is_same<V, i64c>::value) e[u] = sc.exp[l];
+          it.next();
+        }
       }
-      out[o] = v;
-      if (dot_with) dot += v * dot_with[o];
-    };
-    store(zz.x, oa);
-    if (ra + 1 < g.nrows) store(zz.y, oa + g.nx);
+      double ra_[U], rb_[U], va[U], vb[U];
+      if (dot_with) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          ra_[u] = ina[u] ? dot_with[oa[u]] : 0.0;
+          rb_[u] = inb[u] ? dot_with[oa[u] + g.nx] : 0.0;
+        }
+      }
+      if constexpr (std::is_same<V, float2>::value) {
+        float fa[U], fb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          fa[u] = z[u].x;
+          fb[u] = z[u].y;
+        }
+        if (out_scale32) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            fa[u] *= ina[u] ? out_scale32[oa[u]] : 0.f;
+            fb[u] *= inb[u] ? out_scale32[oa[u] + g.nx] : 0.f;
+          }
+        } else if (out_scale) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            fa[u] *= ina[u] ? d2f_rn(out_scale[oa[u]]) : 0.f;
+            fb[u] *= inb[u] ? d2f_rn(out_scale[oa[u] + g.nx]) : 0.f;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          va[u] = f2d(fa[u]);
+          vb[u] = f2d(fb[u]);
+        }
+        if (want_wsum) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) wsum += (ina[u] ? f2d(z[u].x) : 0.0) + (inb[u] ? f2d(z[u].y) : 0.0);
+        }
+      } else {
+        double sa[U], sb[U];
+        if (out_scale) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            sa[u] = ina[u] ? out_scale[oa[u]] : 0.0;
+            sb[u] = inb[u] ? out_scale[oa[u] + g.nx] : 0.0;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          va[u] = ina[u] ? unscaled<V>(z[u].x, e[u]) : 0.0;
+          vb[u] = inb[u] ? unscaled<V>(z[u].y, e[u]) : 0.0;
+        }
+        if (want_wsum) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) wsum += va[u] + vb[u];
+        }
+        if (out_scale) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            va[u] *= sa[u];
+            vb[u] *= sb[u];
+          }
+        }
+      }
+      if (dot_with) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (ina[u]) dot += va[u] * ra_[u];
+          if (inb[u]) dot += vb[u] * rb_[u];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (ina[u]) out[oa[u]] = va[u];
+        if (inb[u]) out[oa[u] + g.nx] = vb[u];
+      }
+    }
   }
-  if (dot_with && b.st)
-    if (grid_reduce(dot, b.partials + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_VR],
-                    &b.st[slot].vr) && threadIdx.x == 0)
-      b.st[slot].vdone = 1;
-  if (want_wsum)
-    grid_reduce(wsum, b.partials2 + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_WSUM],
-                &b.st[slot].wsum);
+  if (b.st) reduce_inverse(b, slot, dot_with != nullptr, dot, want_wsum, wsum);
 }
 
 // ---------------------------------------------------------------------------

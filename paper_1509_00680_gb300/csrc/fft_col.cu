@@ -419,18 +419,16 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, 3>::B)) k_xr_fwd(PassG
   constexpr int R0 = ColPlan<L>::radix(0, false);
   V x[E];
 #pragma unroll
-  for (int q = 0; q < E / R0; ++q)
+  for (int i0 = 0; i0 < E; i0 += 8) {
+    auto all = [](int) { return true; };
+    auto column = [&](int i) { return t + ((i0 + i) / R0) * TPC + ((i0 + i) % R0) * (L / R0); };
+    double a8[8], b8[8];
+    T xa[8], xb[8];
+    load_pairs(in, g.nx, (size_t)ra * g.nx, act, hasb, all, column, a8, b8);
+    scale_pairs<V>(scale, scale32, g.nx, (size_t)ra * g.nx, act, hasb, all, column, red, sum, a8, b8, xa, xb);
 #pragma unroll
-    for (int r = 0; r < R0; ++r) {
-      const int j = t + q * TPC + r * (L / R0);
-      T va = T(0), vb = T(0);
-      if (act && j < g.nx) {
-        const size_t o = (size_t)ra * g.nx + j;
-        va = load_scaled<V>(in, scale, o, red, sum, scale32);
-        if (hasb) vb = load_scaled<V>(in, scale, o + g.nx, red, sum, scale32);
-      }
-      x[q * R0 + r] = mk<V>(va, vb);
-    }
+    for (int i = 0; i < 8; ++i) x[i0 + i] = mk<V>(xa[i], xb[i]);
+  }
   col_stages<V, L, E, -1, false, 0>(x, t, twg + L, line);
   // Z in natural order; Z_k and Z_(L-k) meet through the line
   constexpr int RL = ColPlan<L>::radix(ColPlan<L>::nst - 1, false);
@@ -503,33 +501,13 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, 3>::B)) k_xr_inv(PassG
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
 #pragma unroll
-  for (int q = 0; q < E / RL; ++q)
-#pragma unroll
-    for (int r = 0; r < RL; ++r) {
-      const int j = t + q * TPC + r * (L / RL);
-      if (act && j < g.nx) {
-        const V zz = x[q * RL + r];
-        const size_t oa = (size_t)ra * g.nx + j;
-        const double va = out_value<V>(zz.x, out_scale, oa, out_scale32);
-        out[oa] = va;
-        if (dot_with) dot += va * dot_with[oa];
-        if (want_wsum) wsum += unscaled<V>(zz.x);
-        if (hasb) {
-          const size_t ob = oa + g.nx;
-          const double vb = out_value<V>(zz.y, out_scale, ob, out_scale32);
-          out[ob] = vb;
-          if (dot_with) dot += vb * dot_with[ob];
-          if (want_wsum) wsum += unscaled<V>(zz.y);
-        }
-      }
-    }
-  if (dot_with && b.st)
-    if (grid_reduce(dot, b.partials + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_VR],
-                    &b.st[slot].vr) && threadIdx.x == 0)
-      b.st[slot].vdone = 1;
-  if (want_wsum)
-    grid_reduce(wsum, b.partials2 + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_WSUM],
-                &b.st[slot].wsum);
+  for (int i0 = 0; i0 < E; i0 += 4) {
+    const V z[4] = {x[i0], x[i0 + 1], x[i0 + 2], x[i0 + 3]};
+    auto column = [&](int i) { return t + ((i0 + i) / RL) * TPC + ((i0 + i) % RL) * (L / RL); };
+    store_pairs(z, 0, out, out_scale, out_scale32, dot_with, g.nx, (size_t)ra * g.nx, act, hasb, column, dot,
+                want_wsum, wsum);
+  }
+  if (b.st) reduce_inverse(b, slot, dot_with != nullptr, dot, want_wsum, wsum);
 }
 
 template <typename V, int L>

@@ -239,7 +239,7 @@ constexpr int kThreads = 256;
 // Upper bound on the static shared memory of a spectrum-pass kernel; a
 // launcher opts a kernel in to more dynamic shared memory once dynamic plus
 // this allowance may exceed the default 48 KB per block.
-constexpr size_t kStaticSmemAllowance = 4096;
+constexpr size_t kStaticSmemAllowance = 6144;
 
 
 // Slot served by this block for a spectrum pass of precision V, or -1.
@@ -251,53 +251,206 @@ __device__ __forceinline__ int pass_slot(const Batch& b) {
   return s;
 }
 
-// Input value of the x pass, in * scale: the FP64 product ...
-__device__ __forceinline__ double load_scaled64(const double* in, const double* scale, size_t o, bool red,
-                                                double& sum) {
-  double v = in[o];
-  if (scale) v *= scale[o];
-  if (red) sum += v;
-  return v;
-}
-// ... rounded to the spectrum's real type.  The FP32 spectrum multiplies in
-// FP32 unless the FP64 sum of the products is wanted; conversions run on the
-// integer pipe.
-template <typename V>
-__device__ __forceinline__ typename Real<V>::T load_scaled(const double* in, const double* scale,
-                                                           size_t o, bool red, double& sum,
-                                                           const float* scale32 = nullptr) {
-  if constexpr (std::is_same<V, float2>::value) {
-    if (red) return d2f_rn(load_scaled64(in, scale, o, red, sum));
-    float v = d2f_rn(in[o]);
-    if (scale32) v *= scale32[o];
-    else if (scale) v *= d2f_rn(scale[o]);
-    return v;
-  } else {
-    return df_of(load_scaled64(in, scale, o, red, sum));
+// Rows of an x pass: a[i], b[i] = the values at column(i) of a row (offset row) and of the next
+// one, zero outside the data: all loads of a thread are issued before any is
+// used.
+template <typename S, int N, typename F, typename C>
+__device__ __forceinline__ void load_pairs(const S* __restrict__ src, int nx, size_t row, bool act, bool hasb,
+                                           F ok, C column, S (&a)[N], S (&b)[N]) {
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    a[i] = S(0);
+    b[i] = S(0);
+    if (ok(i)) {
+      const int j = column(i);
+      const bool in = act && j < nx;
+      if (in) a[i] = src[row + j];
+      if (in && hasb) b[i] = src[row + nx + j];
+    }
   }
 }
 
-// Real output value of the x inverse pass as a double (integer-pipe
-// conversions; the FP32 spectrum scales in FP32).  e: exponent of the line
-// (FP64 spectrum only).
+// Input values of an x pass: a, b (loaded from `in`) times the scale factors
+// at the same places, as doubles, and their sum if it is wanted (red) ...
+template <typename V, int N, typename F, typename C>
+__device__ __forceinline__ void scale_pairs(const double* scale, const float* scale32, int nx, size_t row, bool act,
+                                            bool hasb, F ok, C column, bool red, double& sum, const double (&a)[N],
+                                            const double (&b)[N], typename Real<V>::T (&xa)[N],
+                                            typename Real<V>::T (&xb)[N]) {
+  // ... the FP32 spectrum multiplies in FP32 unless the FP64 sum is wanted
+  if constexpr (std::is_same<V, float2>::value) {
+    if (!red) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        xa[i] = d2f_rn(a[i]);
+        xb[i] = d2f_rn(b[i]);
+      }
+      if (scale32) {
+        float sa[N], sb[N];
+        load_pairs(scale32, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          xa[i] *= sa[i];
+          xb[i] *= sb[i];
+        }
+      } else if (scale) {
+        double sa[N], sb[N];
+        load_pairs(scale, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          xa[i] *= d2f_rn(sa[i]);
+          xb[i] *= d2f_rn(sb[i]);
+        }
+      }
+      return;
+    }
+  }
+  double va[N], vb[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    va[i] = a[i];
+    vb[i] = b[i];
+  }
+  if (scale) {
+    double sa[N], sb[N];
+    load_pairs(scale, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (ok(i)) {
+        va[i] *= sa[i];
+        vb[i] *= sb[i];
+      }
+  }
+  if (red) {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (ok(i)) sum += va[i] + vb[i];
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if constexpr (std::is_same<V, float2>::value) {
+      xa[i] = d2f_rn(va[i]);
+      xb[i] = d2f_rn(vb[i]);
+    } else {
+      xa[i] = ok(i) ? df_of(va[i]) : df(0.f, 0.f);
+      xb[i] = ok(i) ? df_of(vb[i]) : df(0.f, 0.f);
+    }
+  }
+}
+
+// Real value of a spectrum line as a double (integer-pipe conversions).  e:
+// exponent of the line (FP64 spectrum only).
 template <typename V>
 __device__ __forceinline__ double unscaled(typename Real<V>::T z, int e = 0) {
   if constexpr (std::is_same<V, float2>::value) return f2d(z);
   else if constexpr (std::is_same<V, dfc>::value) return dbl_of(z);
   else return fx_to_double(z.v, e);
 }
-template <typename V>
-__device__ __forceinline__ double out_value(typename Real<V>::T z, const double* scale, size_t o,
-                                            const float* scale32 = nullptr) {
+
+// Results of an x inverse pass: v = z scale (the FP32 spectrum scales in
+// FP32) to out, (v, r) into dot and the sum of z into wsum where they are
+// wanted, for the N elements x at column(i) of a row pair.  The scale factors
+// and r are loaded before anything is stored: with a load, a product and a
+// store per element the pass waited for HBM once per element (periodic
+// 128^3, FP64 spectrum, with the same change in the forward pass: x passes 98
+// -> 74 us).
+template <typename V, int N, typename C>
+__device__ __forceinline__ void store_pairs(const V (&x)[N], int e, double* __restrict__ out,
+                                            const double* __restrict__ scale, const float* __restrict__ scale32,
+                                            const double* __restrict__ dot_with, int nx, size_t row, bool act,
+                                            bool hasb, C column, double& dot, bool want_wsum, double& wsum) {
+  auto ok = [&](int) { return true; };
+  double va[N], vb[N], ra[N], rb[N];
+  if (dot_with) load_pairs(dot_with, nx, row, act, hasb, ok, column, ra, rb);
   if constexpr (std::is_same<V, float2>::value) {
-    float v = z;
-    if (scale32) v *= scale32[o];
-    else if (scale) v *= d2f_rn(scale[o]);
-    return f2d(v);
+    float fa[N], fb[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      fa[i] = x[i].x;
+      fb[i] = x[i].y;
+    }
+    if (scale32) {
+      float sa[N], sb[N];
+      load_pairs(scale32, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        fa[i] *= sa[i];
+        fb[i] *= sb[i];
+      }
+    } else if (scale) {
+      double sa[N], sb[N];
+      load_pairs(scale, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        fa[i] *= d2f_rn(sa[i]);
+        fb[i] *= d2f_rn(sb[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      va[i] = f2d(fa[i]);
+      vb[i] = f2d(fb[i]);
+    }
+    if (want_wsum) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const bool in = act && column(i) < nx;
+        if (in) wsum += f2d(x[i].x);
+        if (in && hasb) wsum += f2d(x[i].y);
+      }
+    }
   } else {
-    double v = unscaled<V>(z);
-    if (scale) v *= scale[o];
-    return v;
+    double sa[N], sb[N];
+    if (scale) load_pairs(scale, nx, row, act, hasb, ok, column, sa, sb);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const bool in = act && column(i) < nx;
+      va[i] = in ? unscaled<V>(x[i].x, e) : 0.0;
+      vb[i] = in && hasb ? unscaled<V>(x[i].y, e) : 0.0;
+    }
+    if (want_wsum) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) wsum += va[i] + vb[i];
+    }
+    if (scale) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        va[i] *= sa[i];
+        vb[i] *= sb[i];
+      }
+    }
+  }
+  if (dot_with) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const bool in = act && column(i) < nx;
+      if (in) dot += va[i] * ra[i];
+      if (in && hasb) dot += vb[i] * rb[i];
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (act && column(i) < nx) {
+      out[row + column(i)] = va[i];
+      if (hasb) out[row + nx + column(i)] = vb[i];
+    }
+}
+
+// (v, r) and, for the gauge, the sum of w of an x inverse pass (want: the
+// slot projects); the last block flags that v exists.
+__device__ __forceinline__ void reduce_inverse(const Batch& b, int slot, bool want_dot, double dot, bool want_wsum,
+                                               double wsum) {
+  SlotState& S = b.st[slot];
+  double* pd = b.partials + (size_t)slot * b.pstride;
+  if (want_dot && want_wsum) {
+    const double v[2] = {dot, wsum};
+    double* const p[2] = {pd, b.partials2 + (size_t)slot * b.pstride};
+    double* const r[2] = {&S.vr, &S.wsum};
+    if (grid_reduce_k(v, p, &S.counter[CNT_VR], r) && threadIdx.x == 0) S.vdone = 1;
+  } else if (want_dot) {
+    if (grid_reduce(dot, pd, &S.counter[CNT_VR], &S.vr) && threadIdx.x == 0) S.vdone = 1;
+  } else if (want_wsum) {
+    grid_reduce(wsum, pd, &S.counter[CNT_VR], &S.wsum);
   }
 }
 

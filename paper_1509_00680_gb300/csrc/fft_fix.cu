@@ -209,24 +209,29 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_x_fwd(PassGeom g, c
   i64c x[E];
   int e[E];
   auto nonzero = [](int i) { return !HALF || (i % R0) < R0 / 2; };
+  auto column = [&](int i) { return t + (i / R0) * TPC + (i % R0) * (L / R0); };
+  double va[E], vb[E];
+  load_pairs(in, g.nx, (size_t)ra * g.nx, act, hasb, nonzero, column, va, vb);
+  if (scale) {
+    double sa[E], sb[E];
+    load_pairs(scale, g.nx, (size_t)ra * g.nx, act, hasb, nonzero, column, sa, sb);
 #pragma unroll
-  for (int q = 0; q < E / R0; ++q)
+    for (int i = 0; i < E; ++i)
+      if (nonzero(i)) {
+        va[i] *= sa[i];
+        vb[i] *= sb[i];
+      }
+  }
+  if (red) {
 #pragma unroll
-    for (int r = 0; r < R0; ++r) {
-      const int i = q * R0 + r;
-      if (!nonzero(r)) {
-        x[i] = czero<i64c>();
-        continue;
-      }
-      const int j = t + q * TPC + r * (L / R0);
-      double va = 0.0, vb = 0.0;
-      if (act && j < g.nx) {
-        const size_t o = (size_t)ra * g.nx + j;
-        va = load_scaled64(in, scale, o, red, sum);
-        if (hasb) vb = load_scaled64(in, scale, o + g.nx, red, sum);
-      }
-      fx_of_doubles(va, vb, x[i].x.v, x[i].y.v, e[i]);
-    }
+    for (int i = 0; i < E; ++i)
+      if (nonzero(i)) sum += va[i] + vb[i];
+  }
+#pragma unroll
+  for (int i = 0; i < E; ++i) {
+    if (nonzero(i)) fx_of_doubles(va[i], vb[i], x[i].x.v, x[i].y.v, e[i]);
+    else x[i] = czero<i64c>();
+  }
   __syncthreads();
   int rem;
   // one bit free: the unpacking below adds two values
@@ -308,31 +313,14 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_x_inv(PassGeom g, c
   col_stages<i64c, L, E, +1, false, 0>(x, t, twg + L, line, rem);
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
-  auto store = [&](fx z, size_t o) {
-    const double w = fx_to_double(z.v, el);
-    if (want_wsum) wsum += w;
-    const double v = out_scale ? w * out_scale[o] : w;
-    out[o] = v;
-    if (dot_with) dot += v * dot_with[o];
-  };
 #pragma unroll
-  for (int q = 0; q < E / RL; ++q)
-#pragma unroll
-    for (int r = 0; r < RL; ++r) {
-      const int j = t + q * TPC + r * (L / RL);
-      if (act && j < g.nx) {
-        const size_t o = (size_t)ra * g.nx + j;
-        store(x[q * RL + r].x, o);
-        if (hasb) store(x[q * RL + r].y, o + g.nx);
-      }
-    }
-  if (dot_with && b.st)
-    if (grid_reduce(dot, b.partials + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_VR],
-                    &b.st[slot].vr) && threadIdx.x == 0)
-      b.st[slot].vdone = 1;
-  if (want_wsum)
-    grid_reduce(wsum, b.partials2 + (size_t)slot * b.pstride, &b.st[slot].counter[CNT_WSUM],
-                &b.st[slot].wsum);
+  for (int i0 = 0; i0 < E; i0 += 4) {
+    const i64c z[4] = {x[i0], x[i0 + 1], x[i0 + 2], x[i0 + 3]};
+    auto column = [&](int i) { return t + ((i0 + i) / RL) * TPC + ((i0 + i) % RL) * (L / RL); };
+    store_pairs(z, el, out, out_scale, (const float*)nullptr, dot_with, g.nx, (size_t)ra * g.nx, act, hasb, column,
+                dot, want_wsum, wsum);
+  }
+  if (b.st) reduce_inverse(b, slot, dot_with != nullptr, dot, want_wsum, wsum);
 }
 
 template <typename K>

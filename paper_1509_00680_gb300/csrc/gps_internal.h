@@ -45,7 +45,7 @@ enum Phase {
 };
 
 enum Counter {
-  CNT_VR = 0, CNT_PAP, CNT_RR, CNT_AUX, CNT_AUX2, CNT_MU, CNT_WSUM, CNT_AUX3, CNT_APSUM, CNT_PSUM,
+  CNT_VR = 0, CNT_PAP, CNT_RR, CNT_AUX, CNT_AUX2, CNT_MU, CNT_AUX3, CNT_PSUM,
   CNT_COUNT
 };
 

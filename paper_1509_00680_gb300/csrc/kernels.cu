@@ -19,6 +19,7 @@
 // them.  Every reduction is deterministic (fixed-order partials).
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "device_util.cuh"
 #include "gps_internal.h"
@@ -53,6 +54,31 @@ int vec_blocks(size_t n, int nslots) {
 
 #define GRID_STRIDE(i, n) \
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (n); i += (size_t)gridDim.x * blockDim.x)
+
+// The PCG updates work on pairs of neighbouring elements, with 16-byte
+// accesses where every array of the launch allows them (VEC); the pairs and
+// their order of summation are the same either way.
+template <bool VEC>
+__device__ __forceinline__ double2 ld2(const double* __restrict__ p, size_t i) {
+  if (VEC) return *reinterpret_cast<const double2*>(p + i);
+  return make_double2(p[i], p[i + 1]);
+}
+template <bool VEC>
+__device__ __forceinline__ void st2(double* __restrict__ p, size_t i, double2 v) {
+  if (VEC) {
+    *reinterpret_cast<double2*>(p + i) = v;
+  } else {
+    p[i] = v.x;
+    p[i + 1] = v.y;
+  }
+}
+template <typename... P>
+__device__ __forceinline__ bool aligned16(const P*... p) {
+  return ((reinterpret_cast<uintptr_t>(p) | ...) & 15) == 0;
+}
+#define PAIR_STRIDE(i, n)                                                                         \
+  for (size_t i = 2 * (blockIdx.x * (size_t)blockDim.x + threadIdx.x); i + 1 < (n);              \
+       i += 2 * (size_t)gridDim.x * blockDim.x)
 
 #define SLOT_PROLOGUE(b)                  \
   const int slot = batch_slot(b);         \
@@ -334,43 +360,49 @@ __global__ void k_update_p(Batch b, Fields f, size_t n, double inv_n, int period
   const double beta = (S.iter == 0 || S.restart) ? 0.0 : vr / S.vr_prev;
   const double mu4pi = periodic ? kFourPi * S.mu_sum * inv_n : 0.0;
   double acc = 0.0, ap_acc = 0.0, p_acc = 0.0;
-  if (project) {
-#pragma unroll 2
-    GRID_STRIDE(i, n) {
-      const double vi = v[i] - c * s[i];
-      const double av = -qlam[i] * vi - kFourPi * r[i] + mu4pi * sqe[i];
-      const double pi_ = vi + beta * p[i];
-      const double api = av + beta * Ap[i];
-      p[i] = pi_;
-      Ap[i] = api;
-      acc += pi_ * api;
+  // GAUGE: v projected, sums of A p and p; PER: the mean term.  Free, surface
+  // and wire BC: five FP64 operations per point (the FP64 pipe, not HBM, is
+  // the tighter bound of this kernel on GB300).
+  auto one = [&](auto gauge, auto per, double vi, double ri, double qi, double si, double sqi, double& pi_,
+                 double& api) {
+    if (gauge.value) vi -= c * si;
+    double av = -qi * vi - kFourPi * ri;
+    if (per.value) av += mu4pi * sqi;
+    pi_ = vi + beta * pi_;
+    api = av + beta * api;
+    acc += pi_ * api;
+    if (gauge.value) {
       ap_acc += api;
       p_acc += pi_;
     }
+  };
+  auto sweep = [&](auto vec, auto gauge, auto per) {
+    constexpr bool VEC = decltype(vec)::value;
+    const double2 zero = make_double2(0.0, 0.0);
+#pragma unroll 2
+    PAIR_STRIDE(i, n) {
+      const double2 vi = ld2<VEC>(v, i), ri = ld2<VEC>(r, i), qi = ld2<VEC>(qlam, i);
+      const double2 si = gauge.value ? ld2<VEC>(s, i) : zero, sqi = per.value ? ld2<VEC>(sqe, i) : zero;
+      double2 pi_ = ld2<VEC>(p, i), api = ld2<VEC>(Ap, i);
+      one(gauge, per, vi.x, ri.x, qi.x, si.x, sqi.x, pi_.x, api.x);
+      one(gauge, per, vi.y, ri.y, qi.y, si.y, sqi.y, pi_.y, api.y);
+      st2<VEC>(p, i, pi_);
+      st2<VEC>(Ap, i, api);
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+      const size_t i = n - 1;
+      one(gauge, per, v[i], r[i], qlam[i], gauge.value ? s[i] : 0.0, per.value ? sqe[i] : 0.0, p[i], Ap[i]);
+    }
+  };
+  const std::true_type yes{};
+  const std::false_type no{};
+  const bool vec = aligned16(v, r, qlam, s, sqe, p, Ap);
+  if (project) {
+    if (vec) sweep(yes, yes, yes); else sweep(no, yes, yes);
   } else if (periodic) {
-#pragma unroll 2
-    GRID_STRIDE(i, n) {
-      const double vi = v[i];
-      const double av = -qlam[i] * vi - kFourPi * r[i] + mu4pi * sqe[i];
-      const double pi_ = vi + beta * p[i];
-      const double api = av + beta * Ap[i];
-      p[i] = pi_;
-      Ap[i] = api;
-      acc += pi_ * api;
-    }
+    if (vec) sweep(yes, no, yes); else sweep(no, no, yes);
   } else {
-    // free, surface and wire BC: five FP64 operations per point (the FP64
-    // pipe, not HBM, is the tighter bound of this kernel on GB300)
-#pragma unroll 2
-    GRID_STRIDE(i, n) {
-      const double vi = v[i];
-      const double av = -qlam[i] * vi - kFourPi * r[i];
-      const double pi_ = vi + beta * p[i];
-      const double api = av + beta * Ap[i];
-      p[i] = pi_;
-      Ap[i] = api;
-      acc += pi_ * api;
-    }
+    if (vec) sweep(yes, no, no); else sweep(no, no, no);
   }
   bool last;
   if (project)
@@ -419,24 +451,35 @@ __global__ void k_update_r(Batch b, Fields f, size_t n) {
   const double alpha = S.alpha;
   const double m = S.gauge ? S.ap_mean : 0.0;
   double acc = 0.0;
+  // MEAN: the grid mean of A p is removed (and the projected A p kept for the
+  // recurrence)
+  auto one = [&](auto mean, double& xi, double& ri, double pi_, double& api) {
+    xi += alpha * pi_;
+    if (mean.value) api -= m;
+    ri -= alpha * api;
+    acc += ri * ri;
+  };
+  auto sweep = [&](auto vec, auto mean) {
+    constexpr bool VEC = decltype(vec)::value;
+#pragma unroll 2
+    PAIR_STRIDE(i, n) {
+      double2 xi = ld2<VEC>(x, i), ri = ld2<VEC>(r, i), api = ld2<VEC>(Ap, i);
+      const double2 pi_ = ld2<VEC>(p, i);
+      one(mean, xi.x, ri.x, pi_.x, api.x);
+      one(mean, xi.y, ri.y, pi_.y, api.y);
+      st2<VEC>(x, i, xi);
+      st2<VEC>(r, i, ri);
+      if (mean.value) st2<VEC>(Ap, i, api);
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) one(mean, x[n - 1], r[n - 1], p[n - 1], Ap[n - 1]);
+  };
+  const std::true_type yes{};
+  const std::false_type no{};
+  const bool vec = aligned16(x, r, p, Ap);
   if (m != 0.0) {
-#pragma unroll 2
-    GRID_STRIDE(i, n) {
-      x[i] += alpha * p[i];
-      const double api = Ap[i] - m;
-      Ap[i] = api;   // keep the projected A p for the recurrence
-      const double ri = r[i] - alpha * api;
-      r[i] = ri;
-      acc += ri * ri;
-    }
+    if (vec) sweep(yes, yes); else sweep(no, yes);
   } else {
-#pragma unroll 2
-    GRID_STRIDE(i, n) {
-      x[i] += alpha * p[i];
-      const double ri = r[i] - alpha * Ap[i];
-      r[i] = ri;
-      acc += ri * ri;
-    }
+    if (vec) sweep(yes, no); else sweep(no, no);
   }
   if (grid_reduce(acc, slot_partials(b, slot), &S.counter[CNT_RR], &S.rr) && threadIdx.x == 0) {
     S.pdone = 0;
