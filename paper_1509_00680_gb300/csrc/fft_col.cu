@@ -71,20 +71,20 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, MODE>::B)) k_col(PassG
   const V* tw = twg + L;                           // forward-order stage twiddles (global, cached)
   const V* twr = twg + 2 * L;                      // reversed-order stage twiddles (z inverse)
   const int c = threadIdx.x % TC, t = threadIdx.x / TC;
-  const int kx = blockIdx.x * TC + c;
-  const bool act = kx < g.Hx;
+  int kx, outer;
+  const bool act = column_of<MODE>(g, blockIdx.x * TC + c, &kx, &outer);
   V* line = reinterpret_cast<V*>(smem_raw) + c * LS;
   size_t stride;
   V* col;
   int nload, nstore;
   if constexpr (MODE == COL_Z) {
     stride = (size_t)g.Py * g.Hp;
-    col = W + (size_t)blockIdx.y * g.Hp + kx;
+    col = W + (size_t)outer * g.Hp + kx;
     nload = g.nz;
     nstore = g.nz;
   } else {
     stride = g.Hp;
-    col = W + (size_t)blockIdx.y * g.Py * g.Hp + kx;
+    col = W + (size_t)outer * g.Py * g.Hp + kx;
     nload = MODE == COL_Y_FWD ? g.ny : L;    // forward: rows y >= ny are the zero padding
     nstore = MODE == COL_Y_FWD ? L : g.ny;   // inverse: crop to y < ny
   }
@@ -101,13 +101,13 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, MODE>::B)) k_col(PassG
   col_stages<V, L, E, MODE == COL_Y_INV ? +1 : -1, false, 0, HALF>(x, t, tw, line);
   constexpr int RL = ColPlan<L>::radix(ColPlan<L>::nst - 1, false);
   if constexpr (MODE == COL_Z) {
-    const int ky = blockIdx.y;
+    const int ky = act ? outer : 0;
     const int kyp = min(ky, g.Py - ky);
     const int hy = g.Py / 2 + 1;
     const size_t t0 = (size_t)kyp * g.Hx + (act ? kx : 0);
     const size_t tz = (size_t)hy * g.Hx;
     const bool use_k0 = a.slot_k0 && b.st && b.st[slot].use_k0;
-    const bool at0 = use_k0 && kx == 0 && ky == 0;
+    const bool at0 = use_k0 && act && kx == 0 && ky == 0;
 #pragma unroll
     for (int q = 0; q < E / RL; ++q)
 #pragma unroll
@@ -145,7 +145,7 @@ void launch_col_build(const PassGeom& g, const V* tw, const Batch& b, const Pipe
   const size_t sm = (size_t)(TC * line_stride<V>(L)) * sizeof(V);
   if (sm + kStaticSmemAllowance > 48 * 1024)
     cudaFuncSetAttribute(k_col<V, L, MODE, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  const dim3 grid((g.Hx + TC - 1) / TC, MODE == COL_Z ? g.Py : g.nz, nslots);
+  const dim3 grid(column_ctas(g, MODE, TC), 1, nslots);
   count_launch();
   k_col<V, L, MODE, HALF><<<grid, kThreads, sm, st>>>(g, tw, b, a);
 }

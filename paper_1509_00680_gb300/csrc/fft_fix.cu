@@ -102,20 +102,20 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_col(PassGeom g, con
   const i64c* tw = twg + L;                        // forward-order stage twiddles
   const i64c* twr = twg + 2 * L;                   // reversed-order stage twiddles (z inverse)
   const int c = threadIdx.x % TC, t = threadIdx.x / TC;
-  const int kx = blockIdx.x * TC + c;
-  const bool act = kx < g.Hx;
+  int kx, outer;
+  const bool act = column_of<MODE>(g, blockIdx.x * TC + c, &kx, &outer);
   i64c* line = reinterpret_cast<i64c*>(smem_raw) + c * Fix<L>::LS;
   size_t stride;
   i64c* col;
   int nload, nstore;
   if constexpr (MODE == COL_Z) {
     stride = (size_t)g.Py * g.Hp;
-    col = W + (size_t)blockIdx.y * g.Hp + kx;
+    col = W + (size_t)outer * g.Hp + kx;
     nload = g.nz;
     nstore = g.nz;
   } else {
     stride = g.Hp;
-    col = W + (size_t)blockIdx.y * g.Py * g.Hp + kx;
+    col = W + (size_t)outer * g.Py * g.Hp + kx;
     nload = MODE == COL_Y_FWD ? g.ny : L;
     nstore = MODE == COL_Y_FWD ? L : g.ny;
   }
@@ -144,13 +144,13 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_col(PassGeom g, con
   int el = scale_line<L, true>(x, e, nonzero, c, t & 1, 0, sm[0], rem);
   col_stages<i64c, L, E, MODE == COL_Y_INV ? +1 : -1, false, 0, HALF>(x, t, tw, line, rem);
   if constexpr (MODE == COL_Z) {
-    const int ky = blockIdx.y;
+    const int ky = act ? outer : 0;
     const int kyp = min(ky, g.Py - ky);
     const int hy = g.Py / 2 + 1;
     const size_t t0 = (size_t)kyp * g.Hx + (act ? kx : 0);
     const size_t tz = (size_t)hy * g.Hx;
     const bool use_k0 = a.slot_k0 && b.st && b.st[slot].use_k0;
-    const bool at0 = use_k0 && kx == 0 && ky == 0;
+    const bool at0 = use_k0 && act && kx == 0 && ky == 0;
 #pragma unroll
     for (int q = 0; q < E / RL; ++q)
 #pragma unroll
@@ -348,7 +348,7 @@ void launch_col(int mode, const PassGeom& g, const i64c* tw, const Batch& b, con
                 cudaStream_t st) {
   constexpr int TC = Fix<L>::TC;
   const size_t sm = (size_t)TC * Fix<L>::LS * sizeof(i64c);
-  const dim3 grid((g.Hx + TC - 1) / TC, mode == COL_Z ? g.Py : g.nz, nslots);
+  const dim3 grid(column_ctas(g, mode, TC), 1, nslots);
   if (mode == COL_Y_FWD) {
     if (2 * g.ny == L) launch(k_fix_col<L, COL_Y_FWD, true>, grid, sm, g, tw, b, a, st);
     else launch(k_fix_col<L, COL_Y_FWD, false>, grid, sm, g, tw, b, a, st);
