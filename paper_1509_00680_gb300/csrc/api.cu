@@ -2151,8 +2151,7 @@ int gps_v_eps(gps_ctx* ctx, const gps_grid* grid, const double* deps, const doub
   cudaStream_t st = (cudaStream_t)stream;
   GPS_GUARD_BEGIN
   cudaSetDevice(ctx->device);
-  const size_t n = (size_t)grid->nx * grid->ny * grid->nz;
-  launch_veps(stencil16_of(*grid), deps, phi, out, n, st);
+  launch_veps(stencil16_of(*grid), deps, phi, out, st);
   return finish(GPS_OK, st);
   GPS_GUARD_END
 }
@@ -2166,9 +2165,9 @@ int gps_electrostatic_energy(gps_ctx* ctx, const gps_grid* grid, const double* r
   GPS_GUARD_BEGIN
   cudaSetDevice(ctx->device);
   Pool* P = direct_pool(ctx, grid, st);
-  const int nb = dft_blocks(P->n);
+  const int nb = tile_blocks(stencil16_of(*grid));
   if (!P->dft_part) P->dft_part = P->mem.alloc<double>(2 * (size_t)nb);
-  launch_energy(stencil16_of(*grid), rho, eps, phi, P->n, P->dft_part, st);
+  launch_energy(stencil16_of(*grid), rho, eps, phi, P->dft_part, st);
   std::vector<double> part(2 * (size_t)nb);
   ck(cudaMemcpyAsync(part.data(), P->dft_part, part.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   ck(cudaStreamSynchronize(st));

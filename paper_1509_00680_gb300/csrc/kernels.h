@@ -75,10 +75,12 @@ void launch_sccs(const double* rho, double* eps, double* deps, size_t n, double 
 // rho_pol; tmp: n doubles of scratch (ln eps)
 void launch_polarization(const Stencil16& s, const double* rho, const double* eps, const double* phi,
                          double* tmp, double* out, size_t n, cudaStream_t st);
-void launch_veps(const Stencil16& s, const double* deps, const double* phi, double* out, size_t n, cudaStream_t st);
-// part: 2 x dft_blocks(n) doubles, per block sum rho phi and sum eps |grad phi|^2
-void launch_energy(const Stencil16& s, const double* rho, const double* eps, const double* phi, size_t n,
-                   double* part, cudaStream_t st);
+void launch_veps(const Stencil16& s, const double* deps, const double* phi, double* out, cudaStream_t st);
+// blocks (partial sums) of launch_energy
+int tile_blocks(const Stencil16& s);
+// part: 2 x tile_blocks(s) doubles, per block sum rho phi and sum eps |grad phi|^2
+void launch_energy(const Stencil16& s, const double* rho, const double* eps, const double* phi, double* part,
+                   cudaStream_t st);
 
 // ---- comparison solvers (sc.cu): Algorithm 1 (SC), PSD, PSD + DIIS ------
 

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stddef.h>
 
+#include "fix64.cuh"
+
 namespace gps {
 
 struct Stencil16 {
@@ -45,6 +47,140 @@ __device__ __forceinline__ double3 grad16(const double* __restrict__ u, size_t i
              dz);
   }
   return make_double3(dx * s.ihx, dy * s.ihy, dz * s.ihz);
+}
+
+// ---- tiles ------------------------------------------------------------------
+//
+// Derivatives of a field on a tile of 32 x 8 x 8 points (8 along z per thread
+// of a 256-thread block) as 64-bit fixed point.  FP64 issues at 1/64 of the
+// integer rate, so the 48 FP64 operations of grad16 bound every pass that uses
+// it; here a difference is two integer additions and its product with a
+// coefficient three integer multiply-adds, accumulated over the eight
+// distances.  One axis at a time, the values of the tile and of the axis' halo
+// are loaded, brought to the largest magnitude among them (60 bits: 2^-60 of
+// it is the unit, where FP64 rounds each value at 2^-53) and staged in shared
+// memory.  A set with values that are not finite takes FP64 differences.
+// Measured at periodic 128^3: see k_pol.
+struct Tile16 {
+  static constexpr int X = 32, Y = 8, Z = 8, H = 8, T = X * Y;   // points, halo, threads
+  static constexpr int N = X * Y * (Z + 2 * H);                  // most values of an axis (y and z)
+  long long v[N];
+  int top[2];                                                    // largest exponents, in turn
+};
+
+// Q62 digits of a coefficient.
+struct Q62 { int h, l; };
+
+// sum_j d_j (p[j stride] - p[-j stride]) 2^-2, d_j = (-1)^(j+1) (8!)^2 / (j
+// (8-j)! (8+j)!); |values| < 2^60.  The cross products of all eight distances
+// sum to less than 2^63.
+__device__ __forceinline__ long long diff16(const long long* p, int stride) {
+  constexpr Q62 c[8] = {{954437177, -477218588}, {-334053012, 381774871}, {121473823, -2091085088}, {-37960570, 1995641370}, {9344140, 830293600}, {-1668596, -1988966984}, {190697, -1122536352}, {-10429, 1168684963}};
+  unsigned long long hi = 0ull - (1ull << 31), mid = (1ull << 63) + (1ull << 31);
+  const long long *a = p, *b = p;
+#pragma unroll
+  for (int j = 1; j <= 8; ++j) {
+    int h, l;
+    a += stride;
+    b -= stride;
+    digits(*a - *b, h, l);
+    hi += (unsigned long long)mul32(h, c[j - 1].h);
+    mid += (unsigned long long)(mul32(h, c[j - 1].l) + mul32(l, c[j - 1].h));
+  }
+  return (long long)(hi + (mid >> 32));
+}
+
+// Index of position p of an axis of n points, -8 <= p: wrapped, or clamped to
+// the faces; positions past the halo of the last point are not used and read
+// as its end.
+__device__ __forceinline__ int axis16(int p, int n, int per) {
+  p = min(p, n + 7);
+  if (per) return p < 0 ? p + n : p >= n ? p - n : p;
+  return min(max(p, 0), n - 1);
+}
+
+// Derivatives along `axis` (0 x, 1 y, 2 z) of u, without the 1/h, at the
+// thread's points (i0 + tx, j0 + ty, k0 + tz).  turn: 0, 1, 0, .. from call to
+// call; t.top = {0, 0} before the first (and a barrier).  The axis is a
+// run-time argument and the callers loop over it, so that the unrolled
+// conversion and differences exist once (six copies overran the instruction
+// cache: k_pol 270 us).
+__device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, const double* __restrict__ u, int i0, int j0,
+                                             int k0, const Stencil16& s, double (&d)[Tile16::Z]) {
+  constexpr int X = Tile16::X, Y = Tile16::Y, Z = Tile16::Z, H = Tile16::H, XW = X + 2 * H, YW = Y + 2 * H;
+  constexpr int NV = Z + 2 * H;          // values of a thread (x: 2 Z)
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const size_t sy = s.nx, sz = (size_t)s.nx * s.ny;
+  const int ic = min(i0 + tx, s.nx - 1), jc = min(j0 + ty, s.ny - 1);
+  double v[NV];
+  if (axis == 2) {
+    const double* col = u + (size_t)jc * sy + ic;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = col[(size_t)axis16(k0 + q - H, s.nz, s.perz) * sz];
+  } else {
+    // positions of the thread in a plane: three rows (y), or two halves of a row (x)
+    size_t at[3];
+    if (axis == 1) {
+#pragma unroll
+      for (int r = 0; r < 3; ++r) at[r] = (size_t)axis16(j0 + ty + 8 * r - H, s.ny, s.pery) * sy + ic;
+    } else {
+      at[0] = (size_t)jc * sy + axis16(i0 + tx - H, s.nx, s.perx);
+      at[1] = tx < 2 * H ? (size_t)jc * sy + axis16(i0 + tx + X - H, s.nx, s.perx) : at[0];
+      at[2] = at[0];
+    }
+#pragma unroll
+    for (int z = 0; z < Z; ++z) {
+      const double* plane = u + (size_t)min(k0 + z, s.nz - 1) * sz;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) v[3 * z + r] = plane[at[r]];
+    }
+  }
+  int top = 0;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) top = max(top, (__double2hiint(v[q]) >> 20) & 0x7ff);
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (tx == 0) atomicMax(&t.top[turn], top);
+  __syncthreads();                       // also: the previous set has been read
+  top = t.top[turn];
+  if (top == 0x7ff) {
+    __syncthreads();
+    if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
+    const int n = axis == 0 ? s.nx : axis == 1 ? s.ny : s.nz;
+    const int per = axis == 0 ? s.perx : axis == 1 ? s.pery : s.perz;
+    const size_t st = axis == 0 ? 1 : axis == 1 ? sy : sz;
+#pragma unroll
+    for (int tz = 0; tz < Z; ++tz) {
+      const int k = min(k0 + tz, s.nz - 1);
+      const int p = axis == 0 ? ic : axis == 1 ? jc : k;
+      const double* line = u + ((size_t)k * sz + (size_t)jc * sy + ic) - p * st;
+      double a = 0.0;
+      for (int m = 1; m <= 8; ++m)
+        a = fma(s.d[m], line[shift16(p, m, n, per) * st] - line[shift16(p, -m, n, per) * st], a);
+      d[tz] = a;
+    }
+    return;
+  }
+  const int e0 = top + 1024 + 2;         // exponent of the staged values
+  // value 3 z + r goes to first + z step + r part
+  const int first = axis == 0 ? ty * XW + tx : ty * X + tx;
+  const int step = axis == 0 ? Y * XW : axis == 1 ? YW * X : 3 * Y * X;
+  const int part = axis == 0 ? X : Y * X;
+#pragma unroll
+  for (int q = 0; q < NV; ++q) {
+    long long m;
+    int e;
+    fx_of_double(v[q], m, e);
+    m = shift_round(m, e0 - e);
+    const bool put = axis > 0 || q % 3 == 0 || (q % 3 == 1 && tx < 2 * H);
+    if (put) t.v[first + (q / 3) * step + (q % 3) * part] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
+  const int stride = axis == 0 ? 1 : axis == 1 ? X : Y * X;
+  const int next = axis == 0 ? Y * XW : axis == 1 ? YW * X : Y * X;
+  const long long* p = &t.v[first + H * stride];
+#pragma unroll
+  for (int tz = 0; tz < Z; ++tz) d[tz] = fx_to_double(diff16(p + tz * next, stride), e0 + 2);
 }
 
 }  // namespace gps
