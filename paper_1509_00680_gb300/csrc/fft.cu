@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(kThreads) k_x_fwd(PassGeom g, FftSched s, cons
   __syncthreads();
   if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, g.nx, 1, sc);
   const V* res = fft_lines<V, -1, MR, XH>(b0, b1, s, ls, nl, tw, g.nx, sc);
+  pdl_trigger();
   for (LineIter it(g.Hx); it.l < nl; it.next()) {
     const int l = it.l, k = it.j;
     const V* line = res + l * ls;
@@ -456,6 +457,7 @@ __global__ void __launch_bounds__(kThreads) k_y(PassGeom g, FftSched s, const V*
   __syncthreads();
   if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, nload, 0, sc);
   const V* res = fft_lines<V, DIR, MR>(b0, b1, s, ls, nl, tw, nload, sc);
+  pdl_trigger();
   const int nstore = DIR < 0 ? L : g.ny;  // inverse: crop to y < ny
   if (act) {
     const V* line = res + c * ls;
@@ -553,6 +555,7 @@ __global__ void __launch_bounds__(kThreads) k_z(PassGeom g, FftSched s, const V*
   __syncthreads();
   if constexpr (std::is_same<V, i64c>::value) line_scales(res, L, ls, nl, L, 0, sc);
   const V* fin = fft_lines<V, +1, MR, false>(res, other, s, ls, nl, tw, L, sc);
+  pdl_trigger();
   if (act) {
     const V* line = fin + c * ls;
     const int e = std::is_same<V, i64c>::value ? sc.exp[c] : 0;
@@ -627,6 +630,7 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
   __syncthreads();
   if constexpr (std::is_same<V, i64c>::value) line_scales(b0, L, ls, nl, L, 0, sc);
   const V* res = fft_lines<V, +1, MR, false>(b0, b1, s, ls, nl, tw, L, sc);
+  pdl_trigger();
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
   {
@@ -786,10 +790,10 @@ static void x_fwd_mr(const PassGeom& g, const FftSched& s, const V* tw, const Ba
   count_launch();
   if (2 * g.nx == s.L) {
     set_smem(k_x_fwd<V, MR, true>, sm);
-    k_x_fwd<V, MR, true><<<dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_x_fwd<V, MR, true>, dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st, g, s, tw, b, a);
   } else {
     set_smem(k_x_fwd<V, MR, false>, sm);
-    k_x_fwd<V, MR, false><<<dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_x_fwd<V, MR, false>, dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st, g, s, tw, b, a);
   }
 }
 
@@ -828,20 +832,20 @@ void launch_y(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
     if (radix16<V>(s)) {
       if (inverse) {
         set_smem(k_y<V, +1, 16>, sm);
-        k_y<V, +1, 16><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+        launch_pdl(k_y<V, +1, 16>, grid, kThreads, sm, st, g, s, tw, b, a);
       } else {
         set_smem(k_y<V, -1, 16>, sm);
-        k_y<V, -1, 16><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+        launch_pdl(k_y<V, -1, 16>, grid, kThreads, sm, st, g, s, tw, b, a);
       }
       return;
     }
   }
   if (inverse) {
     set_smem(k_y<V, +1, 8>, sm);
-    k_y<V, +1, 8><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_y<V, +1, 8>, grid, kThreads, sm, st, g, s, tw, b, a);
   } else {
     set_smem(k_y<V, -1, 8>, sm);
-    k_y<V, -1, 8><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_y<V, -1, 8>, grid, kThreads, sm, st, g, s, tw, b, a);
   }
 }
 
@@ -857,20 +861,20 @@ void launch_z(const PassGeom& g, const FftSched& s, const V* tw, const Batch& b,
     if (radix16<V>(s)) {
       if (zh) {
         set_smem(k_z<V, 16, true>, sm);
-        k_z<V, 16, true><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+        launch_pdl(k_z<V, 16, true>, grid, kThreads, sm, st, g, s, tw, b, a);
       } else {
         set_smem(k_z<V, 16, false>, sm);
-        k_z<V, 16, false><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+        launch_pdl(k_z<V, 16, false>, grid, kThreads, sm, st, g, s, tw, b, a);
       }
       return;
     }
   }
   if (zh) {
     set_smem(k_z<V, 8, true>, sm);
-    k_z<V, 8, true><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_z<V, 8, true>, grid, kThreads, sm, st, g, s, tw, b, a);
   } else {
     set_smem(k_z<V, 8, false>, sm);
-    k_z<V, 8, false><<<grid, kThreads, sm, st>>>(g, s, tw, b, a);
+    launch_pdl(k_z<V, 8, false>, grid, kThreads, sm, st, g, s, tw, b, a);
   }
 }
 
@@ -883,12 +887,12 @@ void launch_x_inv(const PassGeom& g, const FftSched& s, const V* tw, const Batch
   if constexpr (std::is_same<V, i64c>::value) {
     if (radix16<V>(s)) {
       set_smem(k_x_inv<V, 16>, sm);
-      k_x_inv<V, 16><<<dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st>>>(g, s, tw, b, a);
+      launch_pdl(k_x_inv<V, 16>, dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st, g, s, tw, b, a);
       return;
     }
   }
   set_smem(k_x_inv<V, 8>, sm);
-  k_x_inv<V, 8><<<dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st>>>(g, s, tw, b, a);
+  launch_pdl(k_x_inv<V, 8>, dim3(x_pass_blocks(g), 1, nslots), kThreads, sm, st, g, s, tw, b, a);
 }
 
 #define GPS_INSTANTIATE(V)                                                                       \

@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, MODE>::B)) k_col(PassG
     }
   col_stages<V, L, E, MODE == COL_Y_INV ? +1 : -1, false, 0, HALF>(x, t, tw, line);
   constexpr int RL = ColPlan<L>::radix(ColPlan<L>::nst - 1, false);
+  if constexpr (MODE != COL_Z) pdl_trigger();
   if constexpr (MODE == COL_Z) {
     const int ky = act ? outer : 0;
     const int kyp = min(ky, g.Py - ky);
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, MODE>::B)) k_col(PassG
         x[q * RL + r] = cscale(x[q * RL + r], tv);
       }
     col_stages<V, L, E, +1, true, 0>(x, t, twr, line);
+    pdl_trigger();
     // the reversed transform ends with radix R0
 #pragma unroll
     for (int q = 0; q < E / R0; ++q)
@@ -147,7 +149,7 @@ void launch_col_build(const PassGeom& g, const V* tw, const Batch& b, const Pipe
     cudaFuncSetAttribute(k_col<V, L, MODE, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   const dim3 grid(column_ctas(g, MODE, TC), 1, nslots);
   count_launch();
-  k_col<V, L, MODE, HALF><<<grid, kThreads, sm, st>>>(g, tw, b, a);
+  launch_pdl(k_col<V, L, MODE, HALF>, grid, kThreads, sm, st, g, tw, b, a);
 }
 
 template <typename V, int L, int MODE>
@@ -430,6 +432,7 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, 3>::B)) k_xr_fwd(PassG
     for (int i = 0; i < 8; ++i) x[i0 + i] = mk<V>(xa[i], xb[i]);
   }
   col_stages<V, L, E, -1, false, 0>(x, t, twg + L, line);
+  pdl_trigger();
   // Z in natural order; Z_k and Z_(L-k) meet through the line
   constexpr int RL = ColPlan<L>::radix(ColPlan<L>::nst - 1, false);
 #pragma unroll
@@ -498,6 +501,7 @@ __global__ void __launch_bounds__(kThreads, (ColCfg<V, L, 3>::B)) k_xr_inv(PassG
     }
   col_stages<V, L, E, +1, false, 0>(x, t, twg + L, line);
   constexpr int RL = ColPlan<L>::radix(ColPlan<L>::nst - 1, false);
+  pdl_trigger();
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
 #pragma unroll
@@ -520,10 +524,10 @@ void launch_xr_len(bool inverse, const PassGeom& g, const V* tw, const Batch& b,
   count_launch();
   if (inverse) {
     if (sm + kStaticSmemAllowance > 48 * 1024) cudaFuncSetAttribute(k_xr_inv<V, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_xr_inv<V, L><<<grid, kThreads, sm, st>>>(g, tw, b, a);
+    launch_pdl(k_xr_inv<V, L>, grid, kThreads, sm, st, g, tw, b, a);
   } else {
     if (sm + kStaticSmemAllowance > 48 * 1024) cudaFuncSetAttribute(k_xr_fwd<V, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_xr_fwd<V, L><<<grid, kThreads, sm, st>>>(g, tw, b, a);
+    launch_pdl(k_xr_fwd<V, L>, grid, kThreads, sm, st, g, tw, b, a);
   }
 }
 

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_col(PassGeom g, con
   int rem;
   int el = scale_line<L, true>(x, e, nonzero, c, t & 1, 0, sm[0], rem);
   col_stages<i64c, L, E, MODE == COL_Y_INV ? +1 : -1, false, 0, HALF>(x, t, tw, line, rem);
+  if constexpr (MODE != COL_Z) pdl_trigger();
   if constexpr (MODE == COL_Z) {
     const int ky = act ? outer : 0;
     const int kyp = min(ky, g.Py - ky);
@@ -164,6 +165,7 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_col(PassGeom g, con
       }
     el = scale_line<L, true>(x, e, [](int) { return true; }, c, t & 1, 0, sm[1], rem);
     col_stages<i64c, L, E, +1, true, 0>(x, t, twr, line, rem);
+    pdl_trigger();
     // the reversed transform ends with radix R0
 #pragma unroll
     for (int q = 0; q < E / R0; ++q)
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_x_fwd(PassGeom g, c
   // one bit free: the unpacking below adds two values
   const int el = scale_line<L, false>(x, e, nonzero, l, t & 1, 1, sm, rem);
   col_stages<i64c, L, E, -1, false, 0, HALF>(x, t, twg + L, line, rem);
+  pdl_trigger();
   // Z in natural order; Z_k and Z_(L-k) meet through the line
 #pragma unroll
   for (int q = 0; q < E / RL; ++q)
@@ -311,6 +314,7 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_x_inv(PassGeom g, c
   int rem;
   const int el = scale_line<L, false>(x, e, [](int) { return true; }, l, t & 1, 0, sm, rem);
   col_stages<i64c, L, E, +1, false, 0>(x, t, twg + L, line, rem);
+  pdl_trigger();
   const bool want_wsum = a.red_wsum && b.st && b.st[slot].gauge;
   double dot = 0.0, wsum = 0.0;
 #pragma unroll
@@ -329,7 +333,7 @@ void launch(K kernel, dim3 grid, size_t sm, const PassGeom& g, const i64c* tw, c
   if (sm + kStaticSmemAllowance > 48 * 1024)
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   count_launch();
-  kernel<<<grid, kThreads, sm, st>>>(g, tw, b, a);
+  launch_pdl(kernel, grid, kThreads, sm, st, g, tw, b, a);
 }
 
 template <int L>

@@ -404,6 +404,7 @@ __global__ void k_update_p(Batch b, Fields f, size_t n, double inv_n, int period
   } else {
     if (vec) sweep(yes, no, no); else sweep(no, no, no);
   }
+  pdl_trigger();
   bool last;
   if (project)
     last = grid_reduce3(acc, ap_acc, p_acc, slot_partials(b, slot), slot_partials2(b, slot),
@@ -481,6 +482,7 @@ __global__ void k_update_r(Batch b, Fields f, size_t n) {
   } else {
     if (vec) sweep(yes, no); else sweep(no, no);
   }
+  pdl_trigger();
   if (grid_reduce(acc, slot_partials(b, slot), &S.counter[CNT_RR], &S.rr) && threadIdx.x == 0) {
     S.pdone = 0;
     S.iter += 1;
@@ -805,7 +807,7 @@ __global__ void k_axis_matrix(const double* __restrict__ in, double* __restrict_
 
 void launch_setup_s(const Batch& b, const Fields& f, size_t n, int nslots, cudaStream_t st) {
   count_launch();
-  k_setup_s<<<VEC_GRID(n, nslots)>>>(b, f, n);
+  launch_pdl(k_setup_s, VEC_GRID(n, nslots), b, f, n);
 }
 
 void launch_fd16_q(const Batch& b, const Fields& f, int nx, int ny, int nz, double hx, double hy,
@@ -813,21 +815,21 @@ void launch_fd16_q(const Batch& b, const Fields& f, int nx, int ny, int nz, doub
                    cudaStream_t st) {
   const size_t n = (size_t)nx * ny * nz;
   count_launch();
-  k_fd16_q<<<VEC_GRID(n, nslots)>>>(b, f, nx, ny, nz, 1.0 / (hx * hx), 1.0 / (hy * hy),
+  launch_pdl(k_fd16_q, VEC_GRID(n, nslots), b, f, nx, ny, nz, 1.0 / (hx * hx), 1.0 / (hy * hy),
                                      1.0 / (hz * hz), perx, pery, perz, c);
 }
 
 void launch_setup_final(const Batch& b, const Fields& f, size_t n, double inv_p, int periodic,
                         int nslots, cudaStream_t st) {
   count_launch();
-  k_setup_final<<<VEC_GRID(n, nslots)>>>(b, f, n);
+  launch_pdl(k_setup_final, VEC_GRID(n, nslots), b, f, n);
   count_launch();
   k_setup_phase<<<dim3(1, 1, nslots), 32, 0, st>>>(b, n, inv_p, periodic);
 }
 
 void launch_init(const Batch& b, const Fields& f, size_t n, int nslots, cudaStream_t st) {
   count_launch();
-  k_init<<<VEC_GRID(n, nslots)>>>(b, f, n);
+  launch_pdl(k_init, VEC_GRID(n, nslots), b, f, n);
 }
 
 __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ out, size_t n) {
@@ -842,35 +844,35 @@ void launch_to_float(const double* in, float* out, size_t n, cudaStream_t st) {
 void launch_update_p(const Batch& b, const Fields& f, size_t n, int periodic, int nslots,
                      cudaStream_t st) {
   count_launch();
-  k_update_p<<<VEC_GRID(n, nslots)>>>(b, f, n, 1.0 / (double)n, periodic);
+  launch_pdl(k_update_p, VEC_GRID(n, nslots), b, f, n, 1.0 / (double)n, periodic);
 }
 
 void launch_update_r(const Batch& b, const Fields& f, size_t n, int nslots, cudaStream_t st) {
   count_launch();
-  k_update_r<<<VEC_GRID(n, nslots)>>>(b, f, n);
+  launch_pdl(k_update_r, VEC_GRID(n, nslots), b, f, n);
 }
 
 void launch_nl_eval(const Batch& b, const Fields& f, size_t n, double inv_p, int periodic,
                     int nslots, cudaStream_t st) {
   count_launch();
-  k_nl_eval<<<VEC_GRID(n, nslots)>>>(b, f, n, inv_p, periodic);
+  launch_pdl(k_nl_eval, VEC_GRID(n, nslots), b, f, n, inv_p, periodic);
 }
 
 void launch_nl_step(const Batch& b, const Fields& f, size_t n, int commit, int nslots,
                     cudaStream_t st) {
   count_launch();
-  k_nl_step<<<VEC_GRID(n, nslots)>>>(b, f, n, commit);
+  launch_pdl(k_nl_step, VEC_GRID(n, nslots), b, f, n, commit);
 }
 
 void launch_fp_source(const Batch& b, const Fields& f, size_t n, int nslots, cudaStream_t st) {
   count_launch();
-  k_fp_source<<<VEC_GRID(n, nslots)>>>(b, f, n);
+  launch_pdl(k_fp_source, VEC_GRID(n, nslots), b, f, n);
 }
 
 void launch_fp_residual(const Batch& b, const Fields& f, size_t n, int periodic, int nslots,
                         cudaStream_t st) {
   count_launch();
-  k_fp_residual<<<VEC_GRID(n, nslots)>>>(b, f, n, periodic);
+  launch_pdl(k_fp_residual, VEC_GRID(n, nslots), b, f, n, periodic);
 }
 
 // flag = 1 if a and b differ anywhere (the same-eps test of a warm start).
