@@ -793,6 +793,11 @@ std::map<TuneKey, TuneVal> g_tune;
 int g_radix_order = -1;   // gps_set_radix_order: -1 tunes the radix order, else this one
 int g_x_kernel = -1;      // gps_set_x_kernel: -1 tuned, 0 shared-memory, 1 register-resident (FP32)
 int g_z_kernel = -1;      // gps_set_z_kernel: -1 tuned, 0 plain column kernel, 1 TMA-staged (FP32, df64)
+// Whether any plan of the process uses the TMA-staged z pass (set for good when
+// one is made, so a graph launched later counts too), and waits of that pass
+// that gave up while it was timed as a candidate.
+std::atomic<bool> g_tma_plans{false};
+std::atomic<unsigned int> g_tune_timeouts{0};
 int g_engine_async = 1;   // gps_set_engine_mode: 1 pools advance independently, 0 in lockstep
 
 template <typename F>
@@ -967,6 +972,8 @@ void tune_spec(Shape& S, cudaStream_t st) {
       g.z_tma = 1;
       const float t = time_launch([&] { launch_z<V>(g, best.fz, twz, b, a, 1, st); }, st);
       if (t < tbest || g_z_kernel == 1) { tbest = t; best.g.z_tma = 1; }
+      g_tune_timeouts += take_wait_timeouts();
+      if (best.g.z_tma) g_tma_plans = true;
     }
     ck(cudaStreamSynchronize(st));
     hit = g_tune.emplace(key, best).first;
@@ -1044,7 +1051,9 @@ void launch_round(Pool& P, int m, bool setup, bool init, cudaStream_t st) {
     timed(6, bi, st, [&](const Batch& bb) { launch_update_r(bb, f, n, ns, st); });
   }
   if (P.has_nlpb) {
-    launch_nl_step(batch_of(P, PH_TRIAL, -1), f, n, 0, ns, st);
+    // up to three line-search trials a round: a rejected trial halves the step
+    // and would otherwise cost a round whose PCG launches find nothing to do
+    for (int k = 0; k < 3; ++k) launch_nl_step(batch_of(P, PH_TRIAL, -1), f, n, 0, ns, st);
     launch_nl_step(batch_of(P, PH_COMMIT, -1), f, n, 1, ns, st);
   }
   if (P.has_cert) {
@@ -1524,33 +1533,37 @@ int solve_direct(Pool& P, const double* rho, const double* eps, double* phi, int
   P.has_df64 = s.spec_hi == SPEC_DF64;
   put_active(P, st);
   ensure_tuned(*P.shape, P.has_mixed, P.has_df64, st);
-  // A single GPe / LPB solve runs the pipeline of its current spectrum
-  // precision only (read from the slot state after each round); a switch in
-  // mid-round leaves the rest of that round's iterations without work (the
-  // update kernels wait for their pipeline's flag), the next round runs the
-  // new precision.  Nonlinear PB re-enters the high precision at every outer
-  // step and keeps every pipeline of its pool.
-  const bool hi64 = s.spec_hi == SPEC_FP64, mixed = P.has_mixed;
-  const bool pick = mixed && !P.has_nlpb;
-  if (pick) {
-    P.has_mixed = false;   // the first round starts in the high precision
-  }
-  int m = 2;
+  // A solve runs the pipeline of its current spectrum precision only (read
+  // from the slot state after each round); a switch in mid-round leaves the
+  // rest of that round's iterations without work (the update kernels wait for
+  // their pipeline's flag), the next round runs the new precision.  Nonlinear
+  // PB decides the precision of each inner solve on the device: the round that
+  // starts one launches both pipelines, for two iterations, and a round that
+  // starts with a rejected line-search step launches no PCG iterations.
+  // Measured, free 128^3 nonlinear PB, mixed df64: 371 -> 332 ms against both
+  // pipelines and eight iterations in every round (idle launches cost 2 to 4 us
+  // each, 12 an iteration).
+  const bool hi64 = s.spec_hi == SPEC_FP64, mixed = P.has_mixed, nl = P.has_nlpb;
+  if (mixed && !nl) P.has_mixed = false;   // the first round starts in the high precision
+  int m = 2, iters = 2;
   bool first = true;
   for (;;) {
-    launch_round(P, m, first, first || P.has_nlpb, st);
+    launch_round(P, iters, first, first || nl, st);
     first = false;
     get_states(P, st);
     ck(cudaStreamSynchronize(st));
     if (t_prof) t_prof->resolve();
-    if (P.st_host[0].phase == PH_DONE || P.st_host[0].phase == PH_IDLE) break;
-    if (pick) {
-      const bool lo = P.st_host[0].spec == SPEC_FP32;
-      P.has_mixed = lo;
+    const int phase = P.st_host[0].phase;
+    if (phase == PH_DONE || phase == PH_IDLE) break;
+    if (mixed) {
+      const bool known = !nl || phase == PH_ITER;
+      const bool lo = known && P.st_host[0].spec == SPEC_FP32;
+      P.has_mixed = lo || !known;
       P.has_fp64 = !lo && hi64;
       P.has_df64 = !lo && !hi64;
     }
     if (m < 8) m *= 2;
+    iters = !nl || phase == PH_ITER ? m : phase == PH_TRIAL ? 0 : 2;
   }
   if (keep) {
     const int stt = P.st_host[0].status;
@@ -1759,7 +1772,9 @@ struct ProfScope {
 int finish(int status, cudaStream_t st) {
   if (cudaStreamSynchronize(st) != cudaSuccess) return GPS_ERR_CUDA;
   if (cudaGetLastError() != cudaSuccess) return GPS_ERR_CUDA;
-  if (take_wait_timeouts()) return GPS_ERR_TIMEOUT;   // a bounded device wait gave up
+  // a bounded device wait gave up (the count is read from the device only if
+  // some plan has such waits: the read costs as much as a small kernel)
+  if (g_tune_timeouts.exchange(0) || (g_tma_plans && take_wait_timeouts())) return GPS_ERR_TIMEOUT;
   return status;
 }
 
