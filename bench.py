@@ -136,6 +136,10 @@ FP32_PEAK_TINST = 152 * 128 * 2.070e9 / 1e12
 # parts (8), a product the TwoProd of the high parts by FMA plus the two cross
 # terms (4).
 DF64_ADD_INST, DF64_MUL_INST = 8, 4
+# Integer instructions per operation of the FP64 spectrum passes, which run in
+# 64-bit fixed point: an addition is two, a product three 32 x 32 multiply-adds
+# and about four of splitting and joining its digits.
+FIX64_ADD_INST, FIX64_MUL_INST = 2, 7
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of a kernel from one
 # ncu capture, valid only for the kernel source it was taken with (the SHA-256
@@ -996,7 +1000,7 @@ def gpe_oracle_sample(p, iters):
 def run_fp64_peak(args):
     """Measured FP64 rate of this GPU: a cuBLAS DGEMM (torch.matmul, FP64,
     8192^3, 2 N^3 flops, best of 5 after 2 warm-ups), for comparison with
-    the derived FP64-pipe peak used by the roofline."""
+    the derived FP64-pipe peak."""
     import torch
     n = 8192
     a = torch.randn(n, n, dtype=torch.float64, device="cuda")
@@ -1078,13 +1082,14 @@ def kernel_roofline(kind, ms, P, peaks_, periodic=False):
         if kind.endswith(suf):
             base, prec = kind[:-len(suf)], suf[1:]
     if base in ("x_fwd", "y_fwd", "z", "y_inv", "x_inv") and prec == "fp64":
-        fl = kernel_flops(base, P)
-        ach = fl / (ms / 1e3) / 1e12
-        return {"kernel": kind, "bound": "alu", "achieved": ach, "peak": FP64_PEAK_TFLOPS,
-                "unit": "TFLOP/s", "frac": ach / FP64_PEAK_TFLOPS, "traffic": ncu_traffic(kind),
+        inst = kernel_flops(base, P) * (0.6 * FIX64_ADD_INST + 0.4 * FIX64_MUL_INST)
+        ach = inst / (ms / 1e3) / 1e12
+        return {"kernel": kind, "bound": "alu", "achieved": ach, "peak": FP32_PEAK_TINST,
+                "unit": "T integer instructions/s", "frac": ach / FP32_PEAK_TINST, "traffic": ncu_traffic(kind),
                 "avg_launch_ms": ms,
-                "peak_source": "derived: 152 SM x 2 DFMA/clk x 2 flop x 2.07 GHz (FP64 pipe, measured by --fp64-peak)",
-                "flops_model": "5 L log2 L per complex FFT of length L (+2 per point for the table)"}
+                "peak_source": "derived: 152 SM x 128 lanes x 2.07 GHz (instruction issue)",
+                "model": "5 L log2 L flops per complex FFT of length L (+2 per point for the table), "
+                         "0.6 x 2 + 0.4 x 7 integer instructions per flop (64-bit fixed point)"}
     if base in ("x_fwd", "y_fwd", "z", "y_inv", "x_inv"):
         byt = pass_bytes(P, 8 if prec == "fp32" else 16)[base]
     else:

@@ -54,7 +54,9 @@ typedef enum {
 /* Arithmetic of the spectrum passes (the vacuum solve inside the
  * preconditioner); every vector, dot product, alpha/beta and the ionic term
  * are FP64 in all modes.
- *   GPS_FP64        FP64 spectrum.
+ *   GPS_FP64        FP64-accurate spectrum: 64-bit block fixed point inside the
+ *                   transforms (the integer pipe issues about 30 times the
+ *                   FP64 rate), 58-bit mantissas with a shared exponent between them.
  *   GPS_MIXED       FP64 spectrum until ||r|| <= mixed_switch ||r_0||, then FP32.
  *                   For nonlinear PB r_0 is the residual of the first outer
  *                   step (4 pi F_0): an inner solve that starts below the
