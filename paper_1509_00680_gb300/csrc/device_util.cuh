@@ -40,11 +40,16 @@ __device__ __forceinline__ df fast_two_sum(float a, float b) {   // |a| >= |b|
 // and at most one product per stage, so lo grows by a few ulps of hi and the
 // norm-wise error bound keeps its u^2 order (tested: df64 spectra match the
 // FP64 oracle to 1e-12).
+// The operations are the rounding intrinsics, which the compiler does not
+// contract: an FMA in place of a product and a sum of an error-free
+// transformation counts the product's rounding error twice, which leaves FP32
+// accuracy (seen once in the radix-2 last stage of a 128-point transform).
+__device__ __forceinline__ float df_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ df operator+(df a, df b) {
-  const float s = a.hi + b.hi;
-  const float bb = s - a.hi;
-  const float e = (a.hi - (s - bb)) + (b.hi - bb);   // TwoSum error of hi parts
-  return df(s, e + (a.lo + b.lo));
+  const float s = __fadd_rn(a.hi, b.hi);
+  const float bb = df_sub(s, a.hi);
+  const float e = __fadd_rn(df_sub(a.hi, df_sub(s, bb)), df_sub(b.hi, bb));   // TwoSum error of hi parts
+  return df(s, __fadd_rn(e, __fadd_rn(a.lo, b.lo)));
 }
 __device__ __forceinline__ df operator-(df a) { return df(-a.hi, -a.lo); }
 __device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
@@ -53,7 +58,7 @@ __device__ __forceinline__ df operator-(df a, df b) { return a + (-b); }
 // terms, so hi + lo is the product to within u^2 |a||b| while lo may exceed
 // half an ulp of hi (by the few ulps that a chain of butterflies adds).
 __device__ __forceinline__ df operator*(df a, df b) {
-  const float p = a.hi * b.hi;
+  const float p = __fmul_rn(a.hi, b.hi);
   float e = fmaf(a.hi, b.hi, -p);                     // TwoProd error
   e = fmaf(a.hi, b.lo, e);
   e = fmaf(a.lo, b.hi, e);
@@ -64,14 +69,14 @@ __device__ __forceinline__ df operator*(df a, df b) {
 // low part (16 FP32 operations against 22 for two products and a sum).
 template <int S>
 __device__ __forceinline__ df df_dot2(df a, df b, df c, df d) {
-  const float p = a.hi * b.hi;
-  const float q = S > 0 ? c.hi * d.hi : -(c.hi * d.hi);
+  const float p = __fmul_rn(a.hi, b.hi);
+  const float q = S > 0 ? __fmul_rn(c.hi, d.hi) : -__fmul_rn(c.hi, d.hi);
   const float e1 = fmaf(a.hi, b.hi, -p);
   const float e2 = S > 0 ? fmaf(c.hi, d.hi, -q) : fmaf(-c.hi, d.hi, -q);
-  const float s = p + q;
-  const float bb = s - p;
-  float lo = (p - (s - bb)) + (q - bb);                // TwoSum error of p + q
-  lo += e1 + e2;
+  const float s = __fadd_rn(p, q);
+  const float bb = df_sub(s, p);
+  float lo = __fadd_rn(df_sub(p, df_sub(s, bb)), df_sub(q, bb));   // TwoSum error of p + q
+  lo = __fadd_rn(lo, __fadd_rn(e1, e2));
   lo = fmaf(a.hi, b.lo, lo);
   lo = fmaf(a.lo, b.hi, lo);
   lo = S > 0 ? fmaf(c.hi, d.lo, lo) : fmaf(-c.hi, d.lo, lo);
