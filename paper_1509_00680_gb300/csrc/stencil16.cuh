@@ -142,9 +142,11 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
   if (tx == 0) atomicMax(&t.top[turn], top);
   __syncthreads();                       // also: the previous set has been read
   top = t.top[turn];
+  // The other word, last read before the barrier above, is cleared here: the
+  // barrier below orders it before the next call's atomicMax.
+  if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
   if (top == 0x7ff) {
     __syncthreads();
-    if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
     const int n = axis == 0 ? s.nx : axis == 1 ? s.ny : s.nz;
     const int per = axis == 0 ? s.perx : axis == 1 ? s.pery : s.perz;
     const size_t st = axis == 0 ? 1 : axis == 1 ? sy : sz;
@@ -175,7 +177,6 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
     if (put) t.v[first + (q / 3) * step + (q % 3) * part] = m;
   }
   __syncthreads();
-  if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
   const int stride = axis == 0 ? 1 : axis == 1 ? X : Y * X;
   const int next = axis == 0 ? Y * XW : axis == 1 ? YW * X : Y * X;
   const long long* p = &t.v[first + H * stride];

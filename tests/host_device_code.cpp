@@ -1,0 +1,31 @@
+// Device headers run on the host (host_cuda.h) for test_host_device_code.py.
+#include <chrono>
+
+#include "host_cuda.h"
+
+#include "stencil16.cuh"
+
+using namespace gps;
+
+static void nap() { std::this_thread::sleep_for(std::chrono::milliseconds(20)); }
+
+// Two derivatives in a row along `axis`, of u0 and of u1, on the tile at the
+// origin, as the passes call them; thread 0 leaves every barrier late.
+extern "C" void derivative_pair(const Stencil16* s, int axis, const double* u0, const double* u1, double* d0,
+                                double* d1) {
+  static Tile16 tile;
+  tile.top[0] = tile.top[1] = 0;
+  host_cuda::after_barrier = [](int t) {
+    if (t == 0) nap();
+  };
+  host_cuda::run_block(Tile16::T, [&] {
+    double a[Tile16::Z], b[Tile16::Z];
+    derivative16(tile, axis, 0, u0, 0, 0, 0, *s, a);
+    derivative16(tile, axis, 1, u1, 0, 0, 0, *s, b);
+    for (int z = 0; z < Tile16::Z; ++z) {
+      d0[z * Tile16::T + threadIdx.x] = a[z];
+      d1[z * Tile16::T + threadIdx.x] = b[z];
+    }
+  });
+  host_cuda::after_barrier = nullptr;
+}
