@@ -166,18 +166,15 @@ __device__ __forceinline__ i64c fx_pack(i64c z, int e) {
   return fx_pack_normalized(re, im, e);
 }
 
-// Mantissa and exponent of a double: v = m 2^(e - kBias), m normalized;
-// subnormals count as zero, infinities and NaN as e = kNaN.
+// Mantissa and exponent of a double: v = m 2^(e - kBias), m normalized unless
+// v is zero or subnormal (exponent of the smallest normal numbers); infinities
+// and NaN as e = kNaN.
 __device__ __forceinline__ void fx_of_double(double v, long long& m, int& e) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(v);
   const int be = (int)((u >> 52) & 0x7ffu);
-  m = (long long)(((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9);
+  m = (long long)(((u & 0xfffffffffffffull) | (be == 0 ? 0ull : 0x10000000000000ull)) << 9);
   if ((long long)u < 0) m = -m;
-  e = be + 1024;
-  if (be == 0) {
-    m = 0;
-    e = 0;
-  }
+  e = max(be, 1) + 1024;
   if (be == 0x7ff) e = kNaN;
 }
 
@@ -192,7 +189,7 @@ __device__ __forceinline__ void fx_of_doubles(double a, double b, long long& re,
 }
 
 // v 2^(e - kBias) as the nearest double (ties away from zero in magnitude;
-// below the smallest normal double: zero).
+// gradual underflow).
 __device__ __forceinline__ double fx_to_double(long long v, int e) {
   if (e >= kNaN) return __longlong_as_double(0x7ff8000000000000ll);
   const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
@@ -202,7 +199,10 @@ __device__ __forceinline__ double fx_to_double(long long v, int e) {
   if (lz >= 64) return __longlong_as_double((long long)sign);
   m <<= lz;                                              // top bit at 63: v = m 2^(e - kBias - lz)
   const int be = e - kBias - lz + 63 + 1023;             // biased exponent of the leading bit
-  if (be <= 0) return __longlong_as_double((long long)sign);
+  if (be <= 0) {                                         // subnormal
+    if (be < -52) return __longlong_as_double((long long)sign);
+    return __longlong_as_double((long long)(sign | (((m >> (11 - be)) + 1ull) >> 1)));
+  }
   if (be >= 0x7ff) return __longlong_as_double((long long)(sign | 0x7ff0000000000000ull));
   const unsigned long long q = (m >> 11) + ((m >> 10) & 1ull);
   return __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + q)));

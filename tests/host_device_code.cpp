@@ -29,3 +29,14 @@ extern "C" void derivative_pair(const Stencil16* s, int axis, const double* u0, 
   });
   host_cuda::after_barrier = nullptr;
 }
+
+// d -> fixed point -> double, with the mantissa shifted down by `drop` bits
+// and the exponent moved by the same and by k.
+extern "C" void fixed_round_trip(const double* d, double* out, int n, int drop, int k) {
+  for (int i = 0; i < n; ++i) {
+    long long m;
+    int e;
+    fx_of_double(d[i], m, e);
+    out[i] = fx_to_double(m >> drop, e + drop + k);
+  }
+}

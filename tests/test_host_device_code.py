@@ -74,3 +74,25 @@ def test_tile_maximum_is_not_lost(lib, axis, finite):
     assert np.abs(d1 - ref).max() <= 1e-14 * np.abs(u1).max()
     if finite:
         assert np.abs(d0 - _derivative(u0, axis)).max() <= 1e-14 * np.abs(u0).max()
+
+
+def test_conversions_underflow_gradually(lib):
+    """Subnormal doubles keep their value, and results below the smallest normal
+    number round to the nearest multiple of 2^-1074, ties away from zero."""
+    rng = np.random.default_rng(33)
+    d = np.concatenate([np.ldexp(rng.integers(1, 1 << 52, 4000).astype(float), -1074), np.ldexp(rng.random(4000), -1022),
+                        [0.0, 5e-324, np.finfo(float).tiny, np.finfo(float).max, 1.0]])
+    d = np.concatenate([d, -d])
+    out = np.zeros_like(d)
+    for drop in (0, 9):
+        lib.fixed_round_trip(_ptr(d), _ptr(out), d.size, drop, 0)
+        assert np.array_equal(out, d)
+    m = rng.integers(1 << 52, 1 << 53, 4000)
+    x = np.ldexp(m.astype(float), -52)
+    got = np.zeros_like(x)
+    for k in range(-1090, -1022):            # x 2^k = m 2^(k - 52): the bits below 2^-1074 go
+        s = min(-1074 - (k - 52), 62)
+        ref = np.ldexp(((m + (1 << (s - 1))) >> s).astype(float), -1074)
+        for sign in (1.0, -1.0):
+            lib.fixed_round_trip(_ptr(sign * x), _ptr(got), x.size, 0, k)
+            assert np.array_equal(got, sign * ref), k
