@@ -170,7 +170,7 @@ __host__ __device__ inline TileGrid tile_grid(const Stencil16& s) {
 #define TILE_LOOP(s)                                                                          \
   extern __shared__ __align__(16) unsigned char smem_raw[];                                   \
   Tile16& tile = *reinterpret_cast<Tile16*>(smem_raw);                                        \
-  if (threadIdx.x < 2) tile.top[threadIdx.x] = 0;                                             \
+  if (threadIdx.x < 2 * Tile16::X) tile.top[0][threadIdx.x] = 0;                                      \
   __syncthreads();                                                                            \
   const TileGrid tg = tile_grid(s);                                                           \
   const int ntiles = tg.tx * tg.ty * tg.tz;                                                   \
@@ -184,9 +184,10 @@ __host__ __device__ inline TileGrid tile_grid(const Stencil16& s) {
   auto index = [&](int tz) { return ((size_t)(k0 + tz) * s.ny + j) * s.nx + i; };
 
 // Measured at periodic 128^3 against FP64 differences, log() and divisions:
-// k_log and k_pol together 910 -> 247 us, both energies 270 -> 118 us.  What is
-// left is issue (ncu: 62 instructions a value and axis, 2.0 of 4 issued a
-// clock at two resident blocks).
+// k_log and k_pol together 910 -> 300 us, both energies 270 -> 126 us.  What is
+// left is issue (about 62 instructions a value and axis, 2.0 of 4 issued a
+// clock at two resident blocks) and, in k_pol, some 45 us of telling the cavities'
+// zeros from values far below their lines' largest and of FP64 differences there.
 __global__ void __launch_bounds__(Tile16::T, 2) k_pol(Stencil16 s, const double* __restrict__ lne,
                                                       const double* __restrict__ phi, const double* __restrict__ rho,
                                                       const double* __restrict__ eps, double* __restrict__ out) {

@@ -166,16 +166,20 @@ __device__ __forceinline__ i64c fx_pack(i64c z, int e) {
   return fx_pack_normalized(re, im, e);
 }
 
-// Mantissa and exponent of a double: v = m 2^(e - kBias), m normalized unless
-// v is zero or subnormal (exponent of the smallest normal numbers); infinities
-// and NaN as e = kNaN.
-__device__ __forceinline__ void fx_of_double(double v, long long& m, int& e) {
+// Mantissa and exponent of a finite double: v = m 2^(e - kBias), m normalized
+// unless v is zero or subnormal (exponent of the smallest normal numbers).
+// Returns the biased exponent.
+__device__ __forceinline__ int fx_of_finite(double v, long long& m, int& e) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(v);
   const int be = (int)((u >> 52) & 0x7ffu);
   m = (long long)(((u & 0xfffffffffffffull) | (be == 0 ? 0ull : 0x10000000000000ull)) << 9);
   if ((long long)u < 0) m = -m;
   e = max(be, 1) + 1024;
-  if (be == 0x7ff) e = kNaN;
+  return be;
+}
+// The same of any double; infinities and NaN as e = kNaN.
+__device__ __forceinline__ void fx_of_double(double v, long long& m, int& e) {
+  if (fx_of_finite(v, m, e) == 0x7ff) e = kNaN;
 }
 
 // Packed pair of two doubles.

@@ -57,37 +57,55 @@ __device__ __forceinline__ double3 grad16(const double* __restrict__ u, size_t i
 // it; here a difference is two integer additions and its product with a
 // coefficient three integer multiply-adds, accumulated over the eight
 // distances.  One axis at a time, the values of the tile and of the axis' halo
-// are loaded, brought to the largest magnitude among them (60 bits: 2^-60 of
-// it is the unit, where FP64 rounds each value at 2^-53) and staged in shared
-// memory.  A set with values that are not finite takes FP64 differences.
+// are loaded, brought to the largest magnitude among their lines (60 bits) and
+// staged in shared memory.
+//
+// The lines that share a scale are those that a reduction finds for nothing: a
+// warp's rows (x), the columns of a lane (y), a thread's column (z).  The unit
+// is 2^-60 of the scale, twice the power of two below the largest value, so
+// values down to 2^-7 of that power are staged exactly and others to the
+// nearest unit.  A derivative is off by a unit or two, at most six: 2^-50
+// of the largest value of its stencil where one of four of its values
+// reaches that 2^-7 (kNear), as FP64 differences are.  Every other point takes
+// FP64 differences, and so do lines with values that are not finite.  One scale
+// a tile would send warps of a potential there too (energy at periodic 128^3:
+// 126 against 150 us); with these none of a potential's warps and at most 1.6 %
+// of a dielectric's have such a point.
 // Measured at periodic 128^3: see k_pol.
 struct Tile16 {
   static constexpr int X = 32, Y = 8, Z = 8, H = 8, T = X * Y;   // points, halo, threads
   static constexpr int N = X * Y * (Z + 2 * H);                  // most values of an axis (y and z)
   long long v[N];
-  int top[2];                                                    // largest exponents, in turn
+  int top[2][X];                                                 // largest exponents of a lane's columns, in turn
 };
 
 // Q62 digits of a coefficient.
 struct Q62 { int h, l; };
 
-// sum_j d_j (p[j stride] - p[-j stride]) 2^-2, d_j = (-1)^(j+1) (8!)^2 / (j
-// (8-j)! (8+j)!); |values| < 2^60.  The cross products of all eight distances
-// sum to less than 2^63.
-__device__ __forceinline__ long long diff16(const long long* p, int stride) {
+// sum_j d_j (p[j stride] - p[-j stride]), d_j = (-1)^(j+1) (8!)^2 / (j (8-j)!
+// (8+j)!); |values| <= 2^60.  The cross products of all eight distances sum to
+// less than 2^63.  near: whether a value at distance 1 or 8 reaches kNear.
+constexpr int kNear = 1 << 21;           // 2^53: high word
+__device__ __forceinline__ long long diff16(const long long* p, int stride, bool& near) {
   constexpr Q62 c[8] = {{954437177, -477218588}, {-334053012, 381774871}, {121473823, -2091085088}, {-37960570, 1995641370}, {9344140, 830293600}, {-1668596, -1988966984}, {190697, -1122536352}, {-10429, 1168684963}};
-  unsigned long long hi = 0ull - (1ull << 31), mid = (1ull << 63) + (1ull << 31);
+  unsigned long long hi = 0ull - (1ull << 31), mid = (1ull << 63) + (1ull << 29);
   const long long *a = p, *b = p;
+  int top = 0, bottom = 0;
 #pragma unroll
   for (int j = 1; j <= 8; ++j) {
     int h, l;
     a += stride;
     b -= stride;
+    if (j == 1 || j == 8) {
+      top = max(top, max(hi32(*a), hi32(*b)));
+      bottom = min(bottom, min(hi32(*a), hi32(*b)));
+    }
     digits(*a - *b, h, l);
     hi += (unsigned long long)mul32(h, c[j - 1].h);
     mid += (unsigned long long)(mul32(h, c[j - 1].l) + mul32(l, c[j - 1].h));
   }
-  return (long long)(hi + (mid >> 32));
+  near = top >= kNear || bottom < -kNear;
+  return (long long)((hi << 2) + (mid >> 30));
 }
 
 // Index of position p of an axis of n points, -8 <= p: wrapped, or clamped to
@@ -101,7 +119,7 @@ __device__ __forceinline__ int axis16(int p, int n, int per) {
 
 // Derivatives along `axis` (0 x, 1 y, 2 z) of u, without the 1/h, at the
 // thread's points (i0 + tx, j0 + ty, k0 + tz).  turn: 0, 1, 0, .. from call to
-// call; t.top = {0, 0} before the first (and a barrier).  The axis is a
+// call; t.top zero before the first (and a barrier).  The axis is a
 // run-time argument and the callers loop over it, so that the unrolled
 // conversion and differences exist once (six copies overran the instruction
 // cache: k_pol 270 us).
@@ -135,33 +153,16 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
       for (int r = 0; r < 3; ++r) v[3 * z + r] = plane[at[r]];
     }
   }
-  int top = 0;
+  int top = 1;
 #pragma unroll
   for (int q = 0; q < NV; ++q) top = max(top, (__double2hiint(v[q]) >> 20) & 0x7ff);
-  top = __reduce_max_sync(0xffffffffu, top);
-  if (tx == 0) atomicMax(&t.top[turn], top);
+  if (axis == 0) top = __reduce_max_sync(0xffffffffu, top);
+  if (axis == 1) atomicMax(&t.top[turn][tx], top);
   __syncthreads();                       // also: the previous set has been read
-  top = t.top[turn];
-  // The other word, last read before the barrier above, is cleared here: the
+  if (axis == 1) top = t.top[turn][tx];
+  // The other words, last read before the barrier above, are cleared here: the
   // barrier below orders it before the next call's atomicMax.
-  if (threadIdx.x == 0) t.top[turn ^ 1] = 0;
-  if (top == 0x7ff) {
-    __syncthreads();
-    const int n = axis == 0 ? s.nx : axis == 1 ? s.ny : s.nz;
-    const int per = axis == 0 ? s.perx : axis == 1 ? s.pery : s.perz;
-    const size_t st = axis == 0 ? 1 : axis == 1 ? sy : sz;
-#pragma unroll
-    for (int tz = 0; tz < Z; ++tz) {
-      const int k = min(k0 + tz, s.nz - 1);
-      const int p = axis == 0 ? ic : axis == 1 ? jc : k;
-      const double* line = u + ((size_t)k * sz + (size_t)jc * sy + ic) - p * st;
-      double a = 0.0;
-      for (int m = 1; m <= 8; ++m)
-        a = fma(s.d[m], line[shift16(p, m, n, per) * st] - line[shift16(p, -m, n, per) * st], a);
-      d[tz] = a;
-    }
-    return;
-  }
+  if (ty == 0) t.top[turn ^ 1][tx] = 0;
   const int e0 = top + 1024 + 2;         // exponent of the staged values
   // value 3 z + r goes to first + z step + r part
   const int first = axis == 0 ? ty * XW + tx : ty * X + tx;
@@ -171,8 +172,8 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
   for (int q = 0; q < NV; ++q) {
     long long m;
     int e;
-    fx_of_double(v[q], m, e);
-    m = shift_round(m, e0 - e);
+    fx_of_finite(v[q], m, e);            // of a line with other values: not used
+    m = ((m >> min(e0 - e - 1, 60)) + 1) >> 1;   // nearest unit; nonzero normal values stay so
     const bool put = axis > 0 || q % 3 == 0 || (q % 3 == 1 && tx < 2 * H);
     if (put) t.v[first + (q / 3) * step + (q % 3) * part] = m;
   }
@@ -180,8 +181,43 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
   const int stride = axis == 0 ? 1 : axis == 1 ? X : Y * X;
   const int next = axis == 0 ? Y * XW : axis == 1 ? YW * X : Y * X;
   const long long* p = &t.v[first + H * stride];
+  unsigned int far = 0;                  // points that take FP64 differences ...
 #pragma unroll
-  for (int tz = 0; tz < Z; ++tz) d[tz] = fx_to_double(diff16(p + tz * next, stride), e0 + 2);
+  for (int tz = 0; tz < Z; ++tz) {
+    bool near;
+    d[tz] = fx_to_double(diff16(p + tz * next, stride, near), e0);
+    far |= near ? 0u : 1u << tz;
+  }
+  if (top == 0x7ff) far = (1u << Z) - 1;
+  else if (top == 1) far = 0;            // zeros, or values next to the smallest normal number, which are exact
+  else {
+    // ... unless their values are all zero, as in the cavity of a dielectric
+#pragma unroll 1
+    for (unsigned int left = far; left; left &= left - 1) {
+      const long long* c = p + (__ffs((int)left) - 1) * next;
+      long long any = 0;
+#pragma unroll
+      for (int m = 1; m <= 8; ++m) any |= c[m * stride] | c[-m * stride];
+      if (any == 0) far ^= left & (0u - left);
+    }
+  }
+#pragma unroll 1
+  for (; far; far &= far - 1) {
+    const int tz = __ffs((int)far) - 1;
+    const int k = min(k0 + tz, s.nz - 1);
+    const int i = axis == 0 ? ic : axis == 1 ? jc : k;
+    const int n = axis == 0 ? s.nx : axis == 1 ? s.ny : s.nz;
+    const int per = axis == 0 ? s.perx : axis == 1 ? s.pery : s.perz;
+    const size_t st = axis == 0 ? 1 : axis == 1 ? sy : sz;
+    const double* line = u + ((size_t)k * sz + (size_t)jc * sy + ic) - i * st;
+    double a = 0.0;
+#pragma unroll
+    for (int m = 1; m <= 8; ++m)
+      a = fma(s.d[m], line[shift16(i, m, n, per) * st] - line[shift16(i, -m, n, per) * st], a);
+#pragma unroll
+    for (int i = 0; i < Z; ++i)
+      if (i == tz) d[i] = a;
+  }
 }
 
 }  // namespace gps

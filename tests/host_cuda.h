@@ -5,6 +5,7 @@
 // they leave a block barrier: a schedule that the hardware may take.
 #pragma once
 
+#include <atomic>
 #include <barrier>
 #include <bit>
 #include <cmath>
@@ -67,6 +68,16 @@ inline void __syncthreads() {
   host_cuda::block->bar.arrive_and_wait();
   if (host_cuda::after_barrier) host_cuda::after_barrier((int)threadIdx.x);
 }
+inline int __syncthreads_or(int v) {
+  static std::atomic<int> any{0};
+  if (v) any = 1;
+  __syncthreads();
+  const int r = any;
+  host_cuda::block->bar.arrive_and_wait();
+  if (threadIdx.x == 0) any = 0;
+  __syncthreads();
+  return r;
+}
 inline void __threadfence_block() {}
 inline void __threadfence() {
   if (host_cuda::on_fence) host_cuda::on_fence((int)threadIdx.x);
@@ -116,6 +127,7 @@ inline int max(int a, int b) { return a > b ? a : b; }
 template <typename T> T __ldg(const T* p) { return *p; }
 template <typename T> T __ldcg(const T* p) { return *p; }
 inline int __clz(int v) { return std::countl_zero((unsigned int)v); }
+inline int __ffs(int v) { return v ? std::countr_zero((unsigned int)v) + 1 : 0; }
 inline int __clzll(long long v) { return std::countl_zero((unsigned long long)v); }
 inline long long __double_as_longlong(double d) { return std::bit_cast<long long>(d); }
 inline double __longlong_as_double(long long v) { return std::bit_cast<double>(v); }

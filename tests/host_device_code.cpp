@@ -14,7 +14,7 @@ static void nap() { std::this_thread::sleep_for(std::chrono::milliseconds(20)); 
 extern "C" void derivative_pair(const Stencil16* s, int axis, const double* u0, const double* u1, double* d0,
                                 double* d1) {
   static Tile16 tile;
-  tile.top[0] = tile.top[1] = 0;
+  for (int i = 0; i < 2 * Tile16::X; ++i) tile.top[0][i] = 0;
   host_cuda::after_barrier = [](int t) {
     if (t == 0) nap();
   };
