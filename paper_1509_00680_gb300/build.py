@@ -16,7 +16,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgps.so")
 SOURCES = ["fft.cu", "fft_col.cu", "fft_fix.cu", "kernels.cu", "sc.cu", "dft.cu", "api.cu", "noalloc.cu"]
 HEADERS = ["gps_internal.h", "device_util.cuh", "kernels.h", "fft_common.cuh", "fft_reg.cuh", "fix64.cuh",
-           "stencil16.cuh", "tma.cuh"]
+           "fixmath.cuh", "stencil16.cuh", "tma.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]

@@ -17,6 +17,7 @@
 #include <cmath>
 
 #include "device_util.cuh"
+#include "fixmath.cuh"
 #include "gps_internal.h"
 #include "kernels.h"
 
@@ -26,87 +27,6 @@ constexpr int kTd = 256;
 
 #define DFT_STRIDE(i, n) \
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (n); i += (size_t)gridDim.x * blockDim.x)
-
-// ln x on the integer pipe (the FP64 log costs about fifty FP64 operations a
-// point).  Argument reduction by a table of reciprocals (Tang, ACM TOMS 16,
-// 1990): x = 2^k m, c ~ 1/m in steps of 2^-10 from the top seven bits of m, r =
-// m c - 1 exactly (|r| <= 2^-7), ln x = k ln 2 - ln c + r S(r) with S(r) = 1 -
-// r/2 + r^2/3 - .. + r^8/9 in 62-bit fixed point.  Within 2^-7 of 1 the sum is
-// r S(r) alone and keeps its relative accuracy.  Below one unit in the last
-// place for 2^-7 <= x < 2^8; other arguments take log().  Measured with k_pol.
-struct LogEntry {
-  int c;            // 2^10 / m
-  long long t;      // -ln(c 2^-10), less ln 2 where k counts the next power; Q59
-};
-__device__ const LogEntry kLog[128] = {
-    {1024, 0ll}, {1012, 6795293840941738ll}, {1004, 11370403191593345ll}, {997, 15403628305985996ll},
-    {989, 20047848811844838ll}, {982, 24142462948686780ll}, {975, 28266369413139536ll},
-    {967, 33015815453761981ll}, {960, 37203924447514676ll}, {953, 41422683753552716ll},
-    {946, 45672545304640874ll}, {940, 49340388552248924ll}, {933, 53649244989726276ll},
-    {926, 57990551431621186ll}, {920, 61737871793117407ll}, {913, 66140757644314386ll},
-    {907, 69941611538978585ll}, {901, 73767692524630402ll}, {895, 77619337715354664ll},
-    {889, 81496891028088367ll}, {883, 85400703366900058ll}, {877, 89331132813551606ll},
-    {871, 93288544824601158ll}, {865, 97273312435318552ll}, {859, 101285816470697740ll},
-    {854, 104651037658125515ll}, {848, 108715407625042972ll}, {843, 112124410772773867ll},
-    {838, 115553693653967752ll}, {832, 119695944427871799ll}, {827, 123170703305002408ll},
-    {822, 126666534226467656ll}, {817, 130183694327584893ll}, {812, 133722445479187459ll},
-    {807, 137283054404625057ll}, {802, 140865792800400014ll}, {797, 144470937460575852ll},
-    {792, 148098770405100622ll}, {787, 151749579012193746ll}, {783, 154686964997433189ll},
-    {778, 158379871619800908ll}, {773, 162096588249429227ll}, {769, 165087312219920620ll},
-    {764, 168847669665622644ll}, {760, 171873717308857462ll}, {755, 175678752591287864ll},
-    {751, 178740968303736654ll}, {747, 181819537715677234ll}, {743, 184914636438564366ll},
-    {738, 188807026327093749ll}, {734, 191939972909774099ll}, {730, 195090039504106524ll},
-    {726, 198257414243499389ll}, {722, -198129856782957177ll}, {718, -194927288810863668ll},
-    {714, -191706829304777818ll}, {710, -188468277234650422ll}, {707, -186027367085322990ll},
-    {703, -182756659007360881ll}, {699, -179467287729531389ll}, {695, -176159039038317590ll},
-    {692, -173665333265017499ll}, {688, -170323522443519508ll}, {684, -166962225734538348ll},
-    {681, -164428328237957248ll}, {677, -161032378786174920ll}, {674, -158472223198572013ll},
-    {670, -155040899065517580ll}, {667, -152453935476487310ll}, {664, -149855310103845996ll},
-    {660, -146372152966907931ll}, {657, -143745903539289286ll}, {654, -141107634621625200ll},
-    {650, -137571054496622079ll}, {647, -134904307633017588ll}, {644, -132225166858762518ll},
-    {641, -129533516432429092ll}, {638, -126829238983691274ll}, {635, -124112215482614698ll},
-    {632, -121382325208219438ll}, {629, -118639445716294862ll}, {626, -115883452806445109ll},
-    {623, -113114220488343011ll}, {620, -110331620947169545ll}, {617, -107535524508215101ll},
-    {614, -104725799600618061ll}, {611, -101902312720215328ll}, {608, -99064928391478589ll},
-    {605, -96213509128509165ll}, {603, -94304696946330400ll}, {600, -91429575014732262ll},
-    {597, -88540041384179551ll}, {594, -85635950847720752ll}, {592, -83691730615882293ll},
-    {589, -80763049876401195ll}, {586, -77819414106614471ll}, {584, -75848606196229526ll},
-    {581, -72879703055389870ll}, {579, -70891905388113654ll}, {576, -67897297343059759ll},
-    {574, -65892214443973355ll}, {571, -62871452497689380ll}, {569, -60848781116186610ll},
-    {566, -57801404403785063ll}, {564, -55760833238325512ll}, {561, -52686368605073562ll},
-    {559, -50627578015647709ll}, {557, -48561408232710466ll}, {554, -45448201283712898ll},
-    {552, -43363349997457029ll}, {550, -41270931176333496ll}, {547, -38117993039345648ll},
-    {545, -36006412831050765ll}, {543, -33887069442768983ll}, {541, -31759905581464755ll},
-    {538, -28554369505136558ll}, {536, -26407399603270641ll}, {534, -24252403627037522ll},
-    {532, -22089321343022463ll}, {530, -19918091837203967ll}, {527, -16645836585335176ll},
-    {525, -14453967966276137ll}, {523, -12253733416183569ll}, {521, -10045068828071886ll},
-    {519, -7827909355255884ll}, {517, -5602189399926745ll}, {512, 0ll}, {512, 0ll}};
-
-__device__ __forceinline__ double fx_log(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int be = (int)(u >> 52);                       // sign included: negative arguments fall through
-  if (be < 1023 - 7 || be >= 1023 + 8) return log(x);
-  const int j = (int)(u >> 45) & 127;
-  const int k = be - 1023 + (j >= 53 ? 1 : 0);
-  const int c = __ldg(&kLog[j].c);
-  const long long t = __ldg(&kLog[j].t);
-  const long long r = (long long)(((u & 0xfffffffffffffull) | 0x10000000000000ull) * (unsigned long long)c) -
-                      (1ll << 62);                     // Q62
-  int h, l;
-  digits(r << 7, h, l);
-  constexpr long long a[9] = {4611686018427387904ll, -2305843009213693952ll, 1537228672809129301ll, -1152921504606846976ll, 922337203685477581ll, -768614336404564651ll, 658812288346769701ll, -576460752303423488ll, 512409557603043100ll};
-  long long s = a[8];
-#pragma unroll
-  for (int i = 7; i >= 0; --i) s = a[i] + ((fx_mul(fx(s), h, l).v + 64) >> 7);
-  if (k == 0 && t == 0) {
-    if (r == 0) return 0.0;
-    const int sh = __clzll((unsigned long long)(r < 0 ? -r : r)) - 2;
-    digits(r << sh, h, l);
-    return fx_to_double(fx_mul(fx(s), h, l).v, kBias - 62 - sh);
-  }
-  const long long v = k * 399572145162582989ll + t + ((fx_mul(fx(s), h, l).v + 512) >> 10);
-  return fx_to_double(v, kBias - 59);
-}
 
 // 1 / x of a positive normal double: the mantissa's reciprocal by two Newton
 // steps in 62-bit fixed point from a float (an FP64 division costs about ten

@@ -192,12 +192,9 @@ __device__ __forceinline__ void fx_of_doubles(double a, double b, long long& re,
   if (e > eb) im = shift_round(im, e - eb);
 }
 
-// v 2^(e - kBias) as the nearest double (ties away from zero in magnitude;
-// gradual underflow).
-__device__ __forceinline__ double fx_to_double(long long v, int e) {
-  if (e >= kNaN) return __longlong_as_double(0x7ff8000000000000ll);
-  const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
-  unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+// m 2^(e - kBias) with the sign bit `sign` as the nearest double (ties away
+// from zero; gradual underflow).
+__device__ __forceinline__ double fx_compose(unsigned long long sign, unsigned long long m, int e) {
   const unsigned int mh = (unsigned int)(m >> 32);
   const int lz = mh ? __clz((int)mh) : 32 + __clz((int)(unsigned int)m);
   if (lz >= 64) return __longlong_as_double((long long)sign);
@@ -210,6 +207,12 @@ __device__ __forceinline__ double fx_to_double(long long v, int e) {
   if (be >= 0x7ff) return __longlong_as_double((long long)(sign | 0x7ff0000000000000ull));
   const unsigned long long q = (m >> 11) + ((m >> 10) & 1ull);
   return __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + q)));
+}
+// v 2^(e - kBias) likewise.
+__device__ __forceinline__ double fx_to_double(long long v, int e) {
+  if (e >= kNaN) return __longlong_as_double(0x7ff8000000000000ll);
+  return fx_compose((unsigned long long)v & 0x8000000000000000ull,
+                    v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v, e);
 }
 
 // Digits and exponent of a table factor: t = (w / 2^62) 2^(e - 1022) with

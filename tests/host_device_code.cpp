@@ -3,6 +3,7 @@
 
 #include "host_cuda.h"
 
+#include "fixmath.cuh"
 #include "stencil16.cuh"
 
 using namespace gps;
@@ -39,4 +40,8 @@ extern "C" void fixed_round_trip(const double* d, double* out, int n, int drop, 
     fx_of_double(d[i], m, e);
     out[i] = fx_to_double(m >> drop, e + drop + k);
   }
+}
+
+extern "C" void fixed_log(const double* x, double* out, int n) {
+  for (int i = 0; i < n; ++i) out[i] = fx_log(x[i]);
 }

@@ -133,3 +133,31 @@ def test_tile_derivatives_follow_their_stencils(lib, axis, kind):
     ref = _derivative(ul, axis)[:8, :8]
     big = np.max([np.abs(np.roll(u, s * j, 2 - axis)) for j in range(1, 9) for s in (-1, 1)], axis=0)[:8, :8]
     assert (np.abs(d - ref) <= 2.0 ** -49 * big).all()
+
+
+def log_arguments(n):
+    """Arguments of the fixed-point logarithm: its whole range, around 1, both
+    sides of the table's interval edges and of the near-1 branch."""
+    rng = np.random.default_rng(34)
+    edges = 1.0 + np.arange(129) / 128.0
+    edges = np.concatenate([np.ldexp(edges, k) for k in range(-7, 8)])
+    edges = np.concatenate([np.nextafter(edges, 0.0), edges, np.nextafter(edges, 1e3)])
+    x = np.concatenate([2.0 ** rng.uniform(-7, 8, n), 1.0 + rng.uniform(-0.02, 0.02, n),
+                        1.0 + rng.choice([-1.0, 1.0], n) * 10.0 ** rng.uniform(-15.9, -1.5, n),
+                        1.0 + 2.0 ** -7 * (1.0 + rng.uniform(0, 0.01, n)), edges])
+    return x[(x >= 2.0 ** -7) & (x < 2.0 ** 8)]
+
+
+def ulp_error(got, exact):
+    """Largest distance from `exact` (extended precision) in units in the last
+    place of the exact value."""
+    ref = np.abs(exact.astype(float))
+    return float(np.max(np.abs(got - exact) / np.spacing(np.where(ref > 0, ref, 1.0))))
+
+
+def test_logarithm(lib):
+    """Every result within one unit in the last place, near 1 in particular."""
+    x = log_arguments(200000)
+    got = np.zeros_like(x)
+    lib.fixed_log(_ptr(x), _ptr(got), x.size)
+    assert ulp_error(got, np.log(x.astype(np.longdouble))) < 1.0
