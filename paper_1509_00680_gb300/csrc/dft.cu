@@ -28,26 +28,6 @@ constexpr int kTd = 256;
 #define DFT_STRIDE(i, n) \
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (n); i += (size_t)gridDim.x * blockDim.x)
 
-// 1 / x of a positive normal double: the mantissa's reciprocal by two Newton
-// steps in 62-bit fixed point from a float (an FP64 division costs about ten
-// FP64 operations); below one unit in the last place.
-__device__ __forceinline__ double fx_recip(double x) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int be = (int)(u >> 52);
-  if (be <= 1 || be >= 2045) return 1.0 / x;           // sign included: negative arguments too
-  const long long m = (long long)(((u & 0xfffffffffffffull) | 0x10000000000000ull) << 9);   // Q61, [1, 2)
-  const float f = __uint_as_float(0x3f800000u | (unsigned int)((u >> 29) & 0x7fffffu));
-  long long r = (long long)__float2uint_rn(__frcp_rn(f) * 2147483648.0f) << 31;               // Q62, [1/2, 1]
-  int h, l;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    digits(r, h, l);
-    const long long d = (1ll << 61) - fx_mul(fx(m), h, l).v;                                   // 1 - m r, Q61
-    r += fx_mul(fx(d), h, l).v << 1;
-  }
-  return fx_to_double(r, kBias - 62 - (be - 1023));
-}
-
 // Bound by the FP64 sincos and exp of the transition region; the logarithm and
 // the divisions run on the integer pipe (periodic 128^3: 137 -> 81 us).
 __global__ void k_sccs(const double* __restrict__ rho, double* __restrict__ eps, double* __restrict__ deps,
@@ -60,12 +40,12 @@ __global__ void k_sccs(const double* __restrict__ rho, double* __restrict__ eps,
     } else if (x <= rmin) {
       e = eps0;
     } else {
-      const double ix = fx_recip(x);
-      const double z = 2.0 * kPi * fx_log(rmax * ix) * inv_lnr;
+      const FxDivisor by_x = fx_divisor(x);
+      const double z = 2.0 * kPi * fx_log(fx_div(rmax, by_x)) * inv_lnr;
       double sz, cz;
       sincos(z, &sz, &cz);
-      e = exp((z - sz) * (1.0 / (2.0 * kPi)) * lne);
-      d = -e * lne * (1.0 - cz) * inv_lnr * ix;
+      e = exp(fx_div(z - sz, fx_pi(1)) * lne);
+      d = fx_div(-e * lne * (1.0 - cz) * inv_lnr, by_x);
     }
     eps[i] = e;
     if (deps) deps[i] = d;
@@ -104,7 +84,7 @@ __host__ __device__ inline TileGrid tile_grid(const Stencil16& s) {
   auto index = [&](int tz) { return ((size_t)(k0 + tz) * s.ny + j) * s.nx + i; };
 
 // Measured at periodic 128^3 against FP64 differences, log() and divisions:
-// k_log and k_pol together 910 -> 300 us, both energies 270 -> 126 us.  What is
+// k_log and k_pol together 910 -> 310 us, both energies 270 -> 126 us.  What is
 // left is issue (about 62 instructions a value and axis, 2.0 of 4 issued a
 // clock at two resident blocks) and, in k_pol, some 45 us of telling the cavities'
 // zeros from values far below their lines' largest and of FP64 differences there.
@@ -132,7 +112,7 @@ __global__ void __launch_bounds__(Tile16::T, 2) k_pol(Stencil16 s, const double*
     for (int tz = 0; tz < Tile16::Z; ++tz)
       if (inside(tz)) {
         const double e = eps[index(tz)];
-        out[index(tz)] = acc[tz] * (1.0 / (4.0 * kPi)) - (e - 1.0) * fx_recip(e) * rho[index(tz)];
+        out[index(tz)] = fx_div(acc[tz], fx_pi(2)) - fx_div(e - 1.0, fx_divisor(e)) * rho[index(tz)];
       }
   }
 }
@@ -169,7 +149,7 @@ __global__ void __launch_bounds__(Tile16::T, 2) k_veps(Stencil16 s, const double
     if (__syncthreads_or(any)) grad_square(tile, phi, i0, j0, k0, turn, s, g2);
 #pragma unroll
     for (int tz = 0; tz < Tile16::Z; ++tz)
-      if (inside(tz)) out[index(tz)] = d[tz] != 0.0 ? -d[tz] * g2[tz] * (1.0 / (8.0 * kPi)) : 0.0;
+      if (inside(tz)) out[index(tz)] = d[tz] != 0.0 ? fx_div(-d[tz] * g2[tz], fx_pi(3)) : 0.0;
   }
 }
 

@@ -95,4 +95,60 @@ __device__ __forceinline__ double fx_log(double x) {
   return fx_compose(neg ? 1ull << 63 : 0ull, neg ? 0ull - v : v, kBias - 64 + q);
 }
 
+// a / b, correctly rounded, on the integer pipe (an FP64 division costs about
+// ten FP64 operations): the reciprocal of b's mantissa by two Newton steps in
+// 62-bit fixed point from a float, the quotient's 53 bits from a product with it,
+// off by at most one, and the exact remainder, which decides.  (With the product
+// alone, or with a product by a rounded reciprocal, a quotient may round the
+// other way.)  Zeros apart, operands and quotients that are not normal numbers
+// take FP64 division.
+struct FxDivisor {
+  double b;
+  unsigned long long m;   // mantissa, 53 bits
+  int h, l;               // digits of 2^52 / m, Q62
+  int e;                  // biased exponent, 0 where FP64 division serves
+};
+
+__device__ __forceinline__ FxDivisor fx_divisor(double b) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(b);
+  FxDivisor d;
+  d.b = b;
+  d.e = (int)(u >> 52) & 0x7ff;
+  d.m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
+  if (d.e == 0x7ff) d.e = 0;
+  const float f = __uint_as_float(0x3f800000u | (unsigned int)((u >> 29) & 0x7fffffu));
+  long long r = (long long)__float2uint_rn(__frcp_rn(f) * 2147483648.0f) << 31;               // [1/2, 1]
+  digits(r, d.h, d.l);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const long long t = (1ll << 61) - fx_mul(fx((long long)(d.m << 9)), d.h, d.l).v;          // 1 - m r, Q61
+    r += fx_mul(fx(t), d.h, d.l).v << 1;
+    digits(r, d.h, d.l);
+  }
+  return d;
+}
+
+// 2^k pi, ready made.
+__device__ __forceinline__ FxDivisor fx_pi(int k) {
+  return FxDivisor{3.14159265358979323846 * (1 << k), 7074237752028440ull, 683565276, -1819212355, 1024 + k};
+}
+
+__device__ __forceinline__ double fx_div(double a, const FxDivisor& d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+  const unsigned long long sign = (u ^ (unsigned long long)__double_as_longlong(d.b)) & 0x8000000000000000ull;
+  const int ea = (int)(u >> 52) & 0x7ff;
+  const unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
+  const int s = m >= d.m ? 52 : 53;                      // quotient m 2^s / d.m in [2^52, 2^53)
+  const int e = ea - d.e + 1023 + 52 - s;
+  if (d.e == 0 || ea == 0 || ea == 0x7ff || e < 1 || e > 2046) {
+    if (d.e != 0 && (u << 1) == 0) return __longlong_as_double((long long)sign);
+    return a / d.b;
+  }
+  unsigned long long q = (unsigned long long)((fx_mul(fx((long long)(m << (s - 44))), d.h, d.l).v + 128) >> 8);
+  const long long rem = (long long)((m << s) - q * d.m);   // modulo 2^64; |rem| < 2^54
+  if (2 * rem > (long long)d.m) ++q;
+  if (2 * rem < -(long long)d.m) --q;
+  return __longlong_as_double((long long)(sign | (((unsigned long long)(e - 1) << 52) + q)));
+}
+
 }  // namespace gps

@@ -45,3 +45,10 @@ extern "C" void fixed_round_trip(const double* d, double* out, int n, int drop, 
 extern "C" void fixed_log(const double* x, double* out, int n) {
   for (int i = 0; i < n; ++i) out[i] = fx_log(x[i]);
 }
+
+extern "C" void fixed_divide(const double* a, const double* b, double* out, int n) {
+  for (int i = 0; i < n; ++i) out[i] = fx_div(a[i], fx_divisor(b[i]));
+}
+extern "C" void fixed_divide_by_pi(const double* a, double* out, int n, int k) {
+  for (int i = 0; i < n; ++i) out[i] = fx_div(a[i], fx_pi(k));
+}

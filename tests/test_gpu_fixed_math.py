@@ -8,7 +8,8 @@ import subprocess
 import numpy as np
 import pytest
 
-from test_host_device_code import log_arguments, ulp_error
+import synth
+from test_host_device_code import division_arguments, log_arguments, same_bits, ulp_error
 
 pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -40,3 +41,27 @@ def test_logarithm(lib):
     assert ulp_error(_on_gpu(lib.run_fixed_log, x), np.log(x.astype(np.longdouble))) < 1.0
     got = _on_gpu(lib.run_fixed_log, np.array([0.0, -1.0, np.inf, np.nan, 1.0]))
     assert got[0] == -np.inf and np.isnan(got[1]) and got[2] == np.inf and np.isnan(got[3]) and got[4] == 0.0
+
+
+def test_division_is_correctly_rounded(lib):
+    a, b = division_arguments(300000)
+    with np.errstate(all="ignore"):
+        assert same_bits(_on_gpu(lib.run_fixed_divide, a, b), a / b)
+
+
+def test_polarization_charge_divides_exactly():
+    """A constant potential leaves -((eps - 1)/eps) rho, whose division IEEE
+    arithmetic fixes; with rho = 1 nothing else rounds."""
+    import torch
+    from paper_1509_00680_gb300 import build
+    build.build()
+    from paper_1509_00680_gb300 import gps
+    g = synth.Grid(32, 24, 20, 0.4, 0.4, 0.4, synth.BC_PERIODIC)
+    eps = 1.0 + 80.0 * np.random.default_rng(36).random(g.npts) ** 3
+    one = torch.ones(g.npts, dtype=torch.float64, device="cuda")
+    out = torch.empty_like(one)
+    ctx = gps.Context(0)
+    ctx.polarization_charge(gps.grid_from(g), one, torch.from_numpy(eps).cuda(), one, out)
+    got = out.cpu().numpy()
+    ctx.close()
+    assert np.array_equal(got, -((eps - 1.0) / eps))

@@ -161,3 +161,35 @@ def test_logarithm(lib):
     got = np.zeros_like(x)
     lib.fixed_log(_ptr(x), _ptr(got), x.size)
     assert ulp_error(got, np.log(x.astype(np.longdouble))) < 1.0
+
+
+def division_arguments(n):
+    """Random mantissas at near and far exponents, quotients of small whole
+    numbers, numbers a few units apart and next to powers of two, and what is not a normal
+    number."""
+    rng = np.random.default_rng(35)
+    a, b = rng.uniform(1, 2, (2, n)) * 2.0 ** rng.integers(-40, 40, (2, n)) * rng.choice([-1.0, 1.0], (2, n))
+    far = np.ldexp(rng.uniform(1, 2, (2, n)), rng.integers(-1070, 1023, (2, n)))
+    whole = rng.integers(-1000, 1000, (2, n)).astype(float)
+    m = rng.integers(1 << 52, 1 << 53, n)
+    close = np.array([m, np.clip(m + rng.integers(-4, 5, n), 1 << 52, (1 << 53) - 1)]).astype(float)
+    edge = np.ldexp(1.0 + rng.integers(-3, 4, (2, n)) * 2.0 ** -52, rng.integers(-3, 4, (2, n)))
+    odd = np.array([0.0, -0.0, 1.0, -3.0, 5e-324, 2.2e-308, 1.7e308, np.inf, -np.inf, np.nan])
+    pairs = np.array([(x, y) for x in odd for y in odd]).T
+    return np.concatenate([(a, b), far, whole, close, edge, pairs], axis=1)
+
+
+def same_bits(x, y):
+    return np.array_equal(x, y, equal_nan=True) and np.array_equal(np.signbit(x)[~np.isnan(x)],
+                                                                  np.signbit(y)[~np.isnan(y)])
+
+
+def test_division_is_correctly_rounded(lib):
+    a, b = np.ascontiguousarray(division_arguments(300000))
+    got = np.zeros_like(a)
+    lib.fixed_divide(_ptr(a), _ptr(b), _ptr(got), a.size)
+    with np.errstate(all="ignore"):
+        assert same_bits(got, a / b)
+        for k in (1, 2, 3):
+            lib.fixed_divide_by_pi(_ptr(a), _ptr(got), a.size, k)
+            assert same_bits(got, a / (2 ** k * np.pi))
