@@ -55,8 +55,8 @@ struct __align__(16) i64c {
 // signed 32 x 32 products.  l = -2^31 is avoided so that -l exists.
 __host__ __device__ inline long long q62_digits(long long w) {
   int l = (int)(unsigned int)(w & 0xffffffffll);
-  if (l == (int)0x80000000) l += 1;
-  const long long h = (w - l) / 4294967296ll;
+  const long long h = (w - l) / 4294967296ll;          // exact
+  if (l == (int)0x80000000) l += 1;                    // off by one unit
   return (long long)(((unsigned long long)h << 32) | (unsigned int)l);
 }
 

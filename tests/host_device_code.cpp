@@ -52,3 +52,11 @@ extern "C" void fixed_divide(const double* a, const double* b, double* out, int 
 extern "C" void fixed_divide_by_pi(const double* a, double* out, int n, int k) {
   for (int i = 0; i < n; ++i) out[i] = fx_div(a[i], fx_pi(k));
 }
+
+extern "C" void fixed_digits(const long long* w, long long* out, int n) {
+  for (int i = 0; i < n; ++i) {
+    const long long d = q62_digits(w[i]);
+    out[i] = (long long)hi32(d) * 4294967296ll + lo32(d);
+    if (lo32(d) == (int)0x80000000) out[i] = 1ll << 63;   // has no negative
+  }
+}

@@ -193,3 +193,15 @@ def test_division_is_correctly_rounded(lib):
         for k in (1, 2, 3):
             lib.fixed_divide_by_pi(_ptr(a), _ptr(got), a.size, k)
             assert same_bits(got, a / (2 ** k * np.pi))
+
+
+def test_factor_digits(lib):
+    """Two signed digits give the factor back; a low digit of -2^31, which has
+    no negative, becomes the next one."""
+    rng = np.random.default_rng(37)
+    k = np.concatenate([np.arange(-6, 7), rng.integers(-(1 << 30) + 1, 1 << 30, 1000)])
+    low = k * (1 << 32) - (1 << 31)
+    w = np.concatenate([low, rng.integers(-(1 << 62), 1 << 62, 20000), [1 << 62, -(1 << 62), 0, (1 << 31) - 1]])
+    out = np.zeros_like(w)
+    lib.fixed_digits(_ptr(w), _ptr(out), w.size)
+    assert np.array_equal(out, w + np.isin(w, low))
