@@ -110,10 +110,13 @@ __device__ __forceinline__ void stage(const V* __restrict__ in, V* __restrict__ 
       } else if (Ns <= short_product(L) && Ns * R > short_product(L)) {
         const int rem = sc.rem[line];
         if (rem > 0) {
+          // ties alternate over the elements that are still to be summed: those of
+          // all j / Ns and r at one k
+          const int p = j / Ns;
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            x[r].x.v = shift_round(x[r].x.v - (r & 1), rem);
-            x[r].y.v = shift_round(x[r].y.v - (r & 1), rem);
+            x[r].x.v = shift_round(x[r].x.v - ((p + r) & 1), rem);
+            x[r].y.v = shift_round(x[r].y.v - ((p + r) & 1), rem);
           }
         }
       }
@@ -595,11 +598,12 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
     LineIter it(g.Hx);
     while (it.l < nl) {
       V A[U], B[U];
-      int dst[U], dstm[U];
+      int dst[U], dstm[U], par[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         dst[u] = -1;
         dstm[u] = -1;
+        par[u] = it.j & 1;
         A[u] = czero<V>();
         B[u] = czero<V>();
         if (it.l < nl) {
@@ -619,7 +623,7 @@ __global__ void __launch_bounds__(kThreads) k_x_inv(PassGeom g, FftSched s, cons
       for (int u = 0; u < U; ++u)
         if (dst[u] >= 0) {
           int e = 0;
-          if constexpr (std::is_same<V, i64c>::value) fx_align(A[u], B[u], e);
+          if constexpr (std::is_same<V, i64c>::value) fx_align(A[u], B[u], e, par[u]);
           const V z = mk<V>(A[u].x - B[u].y, A[u].y + B[u].x);                   // Z = A + i B
           const V zm = mk<V>(A[u].x + B[u].y, B[u].x - A[u].y);                  // conj A + i conj B
           b0[dst[u]] = spec_value(z, e);

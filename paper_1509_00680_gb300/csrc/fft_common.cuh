@@ -35,7 +35,9 @@ __device__ __forceinline__ T mulk(T x) {
 }
 template <typename T>
 __device__ __forceinline__ T halve(T x) {
-  if constexpr (std::is_same<T, fx>::value) return fx((x.v + 1) >> 1);
+  // ties to even: rounded one way, the odd sums of a stage's radix-3 butterflies
+  // would add up
+  if constexpr (std::is_same<T, fx>::value) return fx((x.v + ((x.v >> 1) & 1)) >> 1);
   else return T(0.5) * x;
 }
 template <typename V, int DIR, class C, class S>

@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, Fix<L>::B) k_fix_x_inv(PassGeom g, c
           B.y.v &= 63;
         }
       }
-      fx_align(A, B, e[i]);
+      fx_align(A, B, e[i], t & 1);           // k has the parity of t
       if (mirror) {
         A.y = -A.y;
         B.y = -B.y;

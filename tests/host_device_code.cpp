@@ -3,6 +3,7 @@
 
 #include "host_cuda.h"
 
+#include "fft_common.cuh"
 #include "fixmath.cuh"
 #include "stencil16.cuh"
 
@@ -58,5 +59,38 @@ extern "C" void fixed_digits(const long long* w, long long* out, int n) {
     const long long d = q62_digits(w[i]);
     out[i] = (long long)hi32(d) * 4294967296ll + lo32(d);
     if (lo32(d) == (int)0x80000000) out[i] = 1ll << 63;   // has no negative
+  }
+}
+
+// out[i] = X_1 + X_2 - (2 x_0 - x_1 - x_2) of three-point transforms, real part.
+extern "C" void fixed_radix3(const long long* x, long long* out, int n, int forward) {
+  for (int i = 0; i < n; ++i) {
+    i64c v[3] = {{fx(x[3 * i]), fx(0)}, {fx(x[3 * i + 1]), fx(0)}, {fx(x[3 * i + 2]), fx(0)}};
+    if (forward) Dft<i64c, -1, 3>::run(v);
+    else Dft<i64c, +1, 3>::run(v);
+    out[i] = v[1].x.v + v[2].x.v - (2 * x[3 * i] - x[3 * i + 1] - x[3 * i + 2]);
+  }
+}
+
+// Error, in units, of the second of two packed values where the first's
+// exponent is `shift` higher; i counts positions in a line.
+extern "C" void fixed_align(const long long* m, double* out, int n, int shift) {
+  for (int i = 0; i < n; ++i) {
+    i64c a = fx_pack_normalized(1ll << 61, 0, 2000 + shift), b = fx_pack_normalized(m[i], m[i], 2000);
+    const long long w = packed_man(b.x.v);
+    int e;
+    fx_align(a, b, e, i & 1);
+    out[i] = std::ldexp((double)((b.x.v << (shift + 1)) - w), -(shift + 1));
+  }
+}
+
+// Real part, in units, of x times a factor whose real part is +-1/2, less its
+// exact value.
+extern "C" void fixed_half_product(const long long* x, double* out, int n, int negative) {
+  const long long c = negative ? -(1ll << 61) : 1ll << 61;
+  const i64c w{fx(q62_digits(c)), fx(q62_digits(3993765219463853012ll))};   // sqrt(3)/2
+  for (int i = 0; i < n; ++i) {
+    const i64c p = cmul(i64c{fx(x[i]), fx(0)}, w);
+    out[i] = (double)(2 * p.x.v - (negative ? -x[i] : x[i])) / 2;
   }
 }

@@ -205,3 +205,37 @@ def test_factor_digits(lib):
     out = np.zeros_like(w)
     lib.fixed_digits(_ptr(w), _ptr(out), w.size)
     assert np.array_equal(out, w + np.isin(w, low))
+
+
+@pytest.mark.parametrize("forward", [0, 1])
+def test_radix_3_rounds_to_neither_side(lib, forward):
+    """Half of the sums that a radix-3 butterfly halves are odd: an error of one
+    unit, up or down, whose mean stays within five standard deviations of 0."""
+    n = 200000
+    x = np.random.default_rng(38).integers(-(1 << 58), 1 << 58, 3 * n)
+    out = np.zeros(n, dtype=np.int64)
+    lib.fixed_radix3(_ptr(x), _ptr(out), n, forward)
+    assert np.abs(out).max() <= 1 and abs(out.mean()) <= 5 * np.sqrt(0.5 / n)
+
+
+@pytest.mark.parametrize("shift", [0, 3, 6, 7, 9, 12])
+def test_alignment_rounds_to_neither_side(lib, shift):
+    """A value brought to a larger one's exponent: within half a unit, with a
+    mean within five standard deviations (at most 1/2 unit each) of 0."""
+    n = 200000
+    r = np.random.default_rng(39)
+    m = r.integers(1 << 61, 1 << 62, n) * r.choice([-1, 1], n)
+    out = np.zeros(n)
+    lib.fixed_align(_ptr(m), _ptr(out), n, shift)
+    assert np.abs(out).max() <= 0.5 and abs(out.mean()) <= 5 * 0.5 / np.sqrt(n)
+
+
+@pytest.mark.parametrize("negative", [0, 1])
+def test_half_products_round_to_neither_side(lib, negative):
+    """Real numbers times sixth roots of unity are halves: within one unit, with
+    a mean within five standard deviations (1/2 unit) of 0."""
+    n = 200000
+    x = np.random.default_rng(40).integers(-(1 << 56), 1 << 56, n)
+    out = np.zeros(n)
+    lib.fixed_half_product(_ptr(x), _ptr(out), n, negative)
+    assert np.abs(out).max() <= 1 and abs(out.mean()) <= 5 * 0.5 / np.sqrt(n)
