@@ -229,12 +229,17 @@ __device__ __forceinline__ bool grid_reduce_k(const double (&v)[K], double* cons
 #pragma unroll
   for (int k = 0; k < K; ++k)
     if (wid == k && lane == 0) part[k][linear_block()] = bs;
-  if (wid < K && lane == 0) __threadfence();
+  // The ticket is thread 0's, so the fences around it are too: before it, after
+  // the barrier that makes the other warps' partials known to thread 0, and
+  // after it, before the barrier that passes on what the last ticket saw.
   if (K > 1) __syncthreads();
-  if (threadIdx.x == 0) am_last = atomicAdd(counter, 1u) == num_blocks() - 1;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    am_last = atomicAdd(counter, 1u) == num_blocks() - 1;
+    if (am_last) __threadfence();
+  }
   __syncthreads();
   if (!am_last) return false;
-  __threadfence();
   const unsigned int nb = num_blocks(), bd = blockDim.x;
   double s[K];
 #pragma unroll

@@ -3,6 +3,7 @@
 
 #include "host_cuda.h"
 
+#include "device_util.cuh"
 #include "fft_common.cuh"
 #include "fixmath.cuh"
 #include "stencil16.cuh"
@@ -93,4 +94,33 @@ extern "C" void fixed_half_product(const long long* x, double* out, int n, int n
     const i64c p = cmul(i64c{fx(x[i]), fx(0)}, w);
     out[i] = (double)(2 * p.x.v - (negative ? -x[i] : x[i])) / 2;
   }
+}
+
+// One block's K = 3 grid reduction: out[k] = partial k as a thread that takes
+// the ticket has published it, i.e. at that thread's last fence; later warps
+// leave every barrier late.
+extern "C" void published_partials(double* out) {
+  static double part[3];
+  static unsigned int counter;
+  double seen[3] = {-1.0, -1.0, -1.0}, res[3];
+  for (double& x : part) x = -1.0;
+  counter = 0;
+  gridDim = {2, 1, 1};                   // not the last block
+  host_cuda::after_barrier = [](int t) {
+    if (t >= 32) nap();
+  };
+  host_cuda::on_fence = [&](int t) {
+    if (t == 0) std::memcpy(seen, part, sizeof seen);
+  };
+  host_cuda::on_ticket = [&] { std::memcpy(out, seen, sizeof seen); };
+  host_cuda::run_block(128, [&] {
+    const double v[3] = {1.0, 2.0, 3.0};
+    double* const p[3] = {&part[0], &part[1], &part[2]};
+    double* const r[3] = {&res[0], &res[1], &res[2]};
+    grid_reduce_k(v, p, &counter, r);
+  });
+  host_cuda::after_barrier = nullptr;
+  host_cuda::on_fence = nullptr;
+  host_cuda::on_ticket = nullptr;
+  gridDim = {1, 1, 1};
 }

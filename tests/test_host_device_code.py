@@ -239,3 +239,11 @@ def test_half_products_round_to_neither_side(lib, negative):
     out = np.zeros(n)
     lib.fixed_half_product(_ptr(x), _ptr(out), n, negative)
     assert np.abs(out).max() <= 1 and abs(out.mean()) <= 5 * 0.5 / np.sqrt(n)
+
+
+def test_partials_are_published_before_the_ticket(lib):
+    """What other blocks may rely on when they see a block's ticket is what its
+    thread knew at its last fence: the partials of all warps."""
+    out = np.zeros(3)
+    lib.published_partials(_ptr(out))
+    assert np.array_equal(out, 128.0 * np.arange(1, 4))
