@@ -1,5 +1,5 @@
 // Device helpers shared by the kernels of the library: complex arithmetic on
-// double2/float2 and deterministic block / grid reductions.
+// double-float and float2, and deterministic block / grid reductions.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -10,9 +10,8 @@ namespace gps {
 
 // Double-float number: the unevaluated sum hi + lo of two floats, about 48
 // significant bits.  Arithmetic by error-free transformations (Knuth's
-// TwoSum, FMA-based TwoProd; Dekker's renormalizing Fast2Sum where a
-// normalized value is wanted) runs on the FP32 pipe, which on this GPU
-// issues 64x the FP64 rate.  Neither addition nor multiplication
+// TwoSum, FMA-based TwoProd) runs on the FP32 pipe, which on this GPU issues
+// 64x the FP64 rate.  Neither addition nor multiplication
 // renormalizes its result: hi is the rounded result of the hi parts and lo
 // collects the exact error terms, so each operation's error stays bounded by
 // a small multiple of u^2 (|a| + |b|) or u^2 |a||b| (u = 2^-24), the
@@ -30,10 +29,6 @@ struct df {
   __host__ __device__ explicit operator double() const { return (double)hi + (double)lo; }
 };
 
-__device__ __forceinline__ df fast_two_sum(float a, float b) {   // |a| >= |b|
-  const float s = a + b;
-  return df(s, b - (s - a));
-}
 // Addition without the final renormalization: the TwoSum of the hi parts is
 // exact for any operands, so hi + lo stays the sum to within the rounding of
 // the lo parts.  In the FFT passes an element goes through a few additions

@@ -38,24 +38,20 @@ template <typename V>
 __device__ __forceinline__ typename Real<V>::T table_value(const PipeArgs& a, size_t i) {
   if constexpr (std::is_same<V, float2>::value) {
     return a.table32 ? a.table32[i] : d2f_rn(a.table[i]);
-  } else if constexpr (std::is_same<V, dfc>::value) {
+  } else {
     if (a.tabledf) {
       const float2 h = a.tabledf[i];
       return df(h.x, h.y);
     }
     return df_of(a.table[i]);
-  } else {
-    return a.table[i];
   }
 }
 
 template <typename V>
 __device__ __forceinline__ typename Real<V>::T real_of(double v) {
   if constexpr (std::is_same<V, float2>::value) return d2f_rn(v);
-  else if constexpr (std::is_same<V, dfc>::value) return df_of(v);
-  else return v;
+  else return df_of(v);
 }
-
 
 // HALF (forward y and z passes of zero-padded axes): rows >= L/2 of every
 // column are the padding; they are neither read nor transformed.
