@@ -84,10 +84,11 @@ __host__ __device__ inline TileGrid tile_grid(const Stencil16& s) {
   auto index = [&](int tz) { return ((size_t)(k0 + tz) * s.ny + j) * s.nx + i; };
 
 // Measured at periodic 128^3 against FP64 differences, log() and divisions:
-// k_log and k_pol together 910 -> 310 us, both energies 270 -> 126 us.  What is
+// k_log and k_pol together 910 -> 275 us, both energies 270 -> 126 us.  What is
 // left is issue (about 62 instructions a value and axis, 2.0 of 4 issued a
-// clock at two resident blocks) and, in k_pol, some 45 us of telling the cavities'
-// zeros from values far below their lines' largest and of FP64 differences there.
+// clock at two resident blocks) and some 30 us, in k_pol for the bulk solvent's
+// potential, in each for one of cavities in a solvent, of telling zeros from values far
+// below their lines' largest and of FP64 differences there.
 __global__ void __launch_bounds__(Tile16::T, 2) k_pol(Stencil16 s, const double* __restrict__ lne,
                                                       const double* __restrict__ phi, const double* __restrict__ rho,
                                                       const double* __restrict__ eps, double* __restrict__ out) {

@@ -68,15 +68,18 @@ __device__ __forceinline__ double3 grad16(const double* __restrict__ u, size_t i
 // of the largest value of its stencil where one of four of its values
 // reaches that 2^-7 (kNear), as FP64 differences are.  Every other point takes
 // FP64 differences, and so do lines with values that are not finite.  One scale
-// a tile would send warps of a potential there too (energy at periodic 128^3:
-// 126 against 150 us); with these none of a potential's warps and at most 1.6 %
-// of a dielectric's have such a point.
-// Measured at periodic 128^3: see k_pol.
+// a tile would send warps of a smooth potential there too (energy at periodic 128^3:
+// 126 against 150 us); one a row instead of a warp's rows along x
+// costs more than it saves (k_pol 275 against 286 us).  The points that remain
+// (in a potential of cavities in a solvent 3 % along x, in 9 % of the warps) are
+// dealt to all lanes of their warp, 32 at a time: each lane on its own, a warp
+// took as many turns as its worst lane has points (k_pol 310 -> 275 us, k_veps 149 -> 135).
 struct Tile16 {
   static constexpr int X = 32, Y = 8, Z = 8, H = 8, T = X * Y;   // points, halo, threads
   static constexpr int N = X * Y * (Z + 2 * H);                  // most values of an axis (y and z)
   long long v[N];
   int top[2][X];                                                 // largest exponents of a lane's columns, in turn
+  unsigned char list[Y][X * Z];                                  // points of a warp: lane + 32 tz
 };
 
 // Q62 digits of a coefficient.
@@ -201,23 +204,37 @@ __device__ __forceinline__ void derivative16(Tile16& t, int axis, int turn, cons
       if (any == 0) far ^= left & (0u - left);
     }
   }
+  if (!__any_sync(0xffffffffu, far != 0)) return;
+  // a warp's points 32 at a time, whichever lanes they belong to
+  int at[Z], total = 0;
+#pragma unroll
+  for (int tz = 0; tz < Z; ++tz) {
+    const unsigned int b = __ballot_sync(0xffffffffu, far >> tz & 1);
+    at[tz] = far >> tz & 1 ? total + __popc(b & ((1u << tx) - 1)) : -32;
+    if (far >> tz & 1) t.list[ty][at[tz]] = (unsigned char)(tx + 32 * tz);
+    total += __popc(b);
+  }
+  __syncwarp();
 #pragma unroll 1
-  for (; far; far &= far - 1) {
-    const int tz = __ffs((int)far) - 1;
-    const int k = min(k0 + tz, s.nz - 1);
-    const int i = axis == 0 ? ic : axis == 1 ? jc : k;
+  for (int base = 0; base < total; base += 32) {
+    const int w = t.list[ty][min(base + tx, total - 1)];
+    const int x = min(i0 + (w & 31), s.nx - 1), z = min(k0 + (w >> 5), s.nz - 1);
+    const int i = axis == 0 ? x : axis == 1 ? jc : z;
     const int n = axis == 0 ? s.nx : axis == 1 ? s.ny : s.nz;
     const int per = axis == 0 ? s.perx : axis == 1 ? s.pery : s.perz;
     const size_t st = axis == 0 ? 1 : axis == 1 ? sy : sz;
-    const double* line = u + ((size_t)k * sz + (size_t)jc * sy + ic) - i * st;
+    const double* line = u + ((size_t)z * sz + (size_t)jc * sy + x) - i * st;
     double a = 0.0;
 #pragma unroll
     for (int m = 1; m <= 8; ++m)
       a = fma(s.d[m], line[shift16(i, m, n, per) * st] - line[shift16(i, -m, n, per) * st], a);
 #pragma unroll
-    for (int i = 0; i < Z; ++i)
-      if (i == tz) d[i] = a;
+    for (int tz = 0; tz < Z; ++tz) {
+      const double v = __shfl_sync(0xffffffffu, a, (at[tz] - base) & 31);
+      if (at[tz] >= base && at[tz] < base + 32) d[tz] = v;
+    }
   }
+  __syncwarp();                          // the list has been read
 }
 
 }  // namespace gps

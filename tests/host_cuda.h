@@ -108,6 +108,18 @@ inline int __reduce_max_sync(unsigned, int v) {
     return m;
   });
 }
+inline unsigned int __ballot_sync(unsigned, int v) {
+  return host_warp(v, [](auto at, int) {
+    unsigned int b = 0;
+    for (int l = 0; l < 32; ++l) b |= (at(l) != 0 ? 1u : 0u) << l;
+    return (int)b;
+  });
+}
+inline int __any_sync(unsigned m, int v) { return __ballot_sync(m, v) != 0; }
+template <typename T> T __shfl_sync(unsigned, T v, int from) {
+  return host_warp(v, [&](auto at, int) { return at(from & 31); });
+}
+inline void __syncwarp() { host_cuda::block->warps[threadIdx.x / 32]->bar.arrive_and_wait(); }
 inline int atomicMax(int* p, int v) {
   std::lock_guard<std::mutex> lock(host_cuda::atomics);
   const int old = *p;
@@ -127,6 +139,7 @@ inline int max(int a, int b) { return a > b ? a : b; }
 template <typename T> T __ldg(const T* p) { return *p; }
 template <typename T> T __ldcg(const T* p) { return *p; }
 inline int __clz(int v) { return std::countl_zero((unsigned int)v); }
+inline int __popc(unsigned int v) { return std::popcount(v); }
 inline int __ffs(int v) { return v ? std::countr_zero((unsigned int)v) + 1 : 0; }
 inline int __clzll(long long v) { return std::countl_zero((unsigned long long)v); }
 inline long long __double_as_longlong(double d) { return std::bit_cast<long long>(d); }
