@@ -250,11 +250,12 @@ __device__ __forceinline__ void fx_apply(i64c& z, int& e, double t) {
 __device__ __forceinline__ void fx_align(i64c& a, i64c& b, int& e, int parity) {
   const int ea = packed_exp(a), eb = packed_exp(b);
   const int top = max(ea, eb);
-  const int sa = top - ea + 1, sb = top - eb + 1;
-  a.x.v = shift_round(packed_man(a.x.v) - parity, sa);
-  a.y.v = shift_round(packed_man(a.y.v) - parity, sa);
-  b.x.v = shift_round(packed_man(b.x.v) - parity, sb);
-  b.y.v = shift_round(packed_man(b.y.v) - parity, sb);
+  const int sa = min(top - ea + 1, 63), sb = min(top - eb + 1, 63);
+  const long long ha = (1ll << (sa - 1)) - parity, hb = (1ll << (sb - 1)) - parity;
+  a.x.v = (packed_man(a.x.v) + ha) >> sa;
+  a.y.v = (packed_man(a.y.v) + ha) >> sa;
+  b.x.v = (packed_man(b.x.v) + hb) >> sb;
+  b.y.v = (packed_man(b.y.v) + hb) >> sb;
   e = top >= kNaN ? kNaN : top + 1;
 }
 
