@@ -1277,7 +1277,8 @@ struct Engine {
   // PCG iterations per round: more for small pools, whose iterations are
   // short, so that a round amortizes its host-side state read (and
   // admission) over at least about a millisecond of device work; fewer with
-  // nonlinear-PB slots, whose line-search trials take one round each.
+  // nonlinear-PB slots, whose inner solves end in mid-round and whose rejected
+  // line-search steps beyond three wait for the next round.
   static int round_iters(const Pool& P) {
     if (!g_engine_async) return 4;
     const double pts = (double)P.n * std::max(1, P.busy());

@@ -28,7 +28,7 @@ template <typename V, int L, int MODE> struct ColCfg {
   static constexpr bool f32 = std::is_same<V, float2>::value;
   static constexpr int E = (f32 && L >= 256) ? 16 : 8;
   // Resident CTAs per SM asked of the register allocator: 2 (128 registers a
-  // thread) at 16 elements, 3 (85) otherwise.  Measured: the FP32 z pass at
+  // thread) at 16 elements, 3 (80) otherwise.  Measured: the FP32 z pass at
   // 16 elements takes ~146 registers uncapped, fits one CTA per SM and runs
   // 1.6x slower; the df64 passes gain 2-3 % from the third CTA.
   static constexpr int B = (f32 && E == 16) ? 2 : 3;

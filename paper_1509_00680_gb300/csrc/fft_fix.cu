@@ -20,8 +20,9 @@ namespace {
 
 template <int L> struct Fix {
   static constexpr int E = 8, TPC = L / E, TC = kThreads / TPC, LS = line_stride<i64c>(L);
-  // Resident CTAs per SM asked of the register allocator (85 registers a
-  // thread): the passes are bound by issue and shared-memory exchanges.
+  // Resident CTAs per SM asked of the register allocator (80 registers a
+  // thread; k_fix_x_inv<L, false> spills 48 to 76 bytes at that): the passes
+  // are bound by issue and shared-memory exchanges.
   static constexpr int B = 3;
 };
 

@@ -15,7 +15,7 @@ enum ColMode { COL_Y_FWD = 0, COL_Y_INV = 1, COL_Z = 2 };
 // where tiles of each row would leave 15 of 80 columns idle at Hx = 65 and 31
 // of 64 at Hx = 33.  A row counts Hp columns (Hx rounded up to even), so that
 // tiles start on a 32-byte sector in every row.  Measured, FP64 spectrum: z
-// pass of free 64^3 39 -> 33 us, y pass of periodic 128^3 22.5 -> 19.6 us.
+// pass of free 64^3 39 -> 33 us, y pass of periodic 128^3 22.5 -> 18.7 us.
 template <int MODE>
 __device__ __forceinline__ bool column_of(const PassGeom& g, int id, int* kx, int* outer) {
   *outer = id / g.Hp;
